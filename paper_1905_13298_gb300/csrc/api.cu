@@ -185,6 +185,8 @@ ds_status conv_launch(const int32_t* x, const ds_weights* w, const int32_t* bias
   p.split_acc = split_acc;
   p.split_capacity = split_capacity;
   if (!(flags & DS_CONV_IM2COL)) {
+    if (shift_mma_preferred(&p, 1, true))
+      return cuda_check(launch_shift_mma(&p, 1, true, st), "conv2d_shift (tensor core) launch");
     if (conv_pointwise_supported(p)) return cuda_check(launch_conv2d_pointwise(p, st), "conv2d_shift (pointwise) launch");
     if (conv_direct_supported(p)) return cuda_check(launch_conv2d_direct(p, st), "conv2d_shift (direct) launch");
   }
@@ -193,6 +195,7 @@ ds_status conv_launch(const int32_t* x, const ds_weights* w, const int32_t* bias
 }
 
 size_t conv_split_bytes(const GemmParams& p) {
+  if (shift_mma_preferred(&p, 1, true)) return 0;
   if (conv_pointwise_supported(p)) return conv_pointwise_split_bytes(p);
   return conv_direct_split_bytes(p);
 }
@@ -200,6 +203,8 @@ size_t conv_split_bytes(const GemmParams& p) {
 // LinearShift kernel choice: small batches split the reduction over a
 // thread-block cluster, large ones run the 128 x 64-tile shift GEMM.
 static ds_status launch_fc(const GemmParams& p, cudaStream_t st) {
+  if (shift_mma_preferred(&p, 1, false))
+    return cuda_check(launch_shift_mma(&p, 1, false, st), "linear_shift (tensor core) launch");
   if (linear_cluster_preferred(p)) return cuda_check(launch_linear_cluster(p, st), "linear_shift (cluster) launch");
   return cuda_check(launch_linear_shift(p, st), "linear_shift launch");
 }
@@ -423,7 +428,10 @@ ds_status ds_linear_shift_bf16(const uint16_t* x, const ds_weights* w, const flo
                     "linear_shift_bf16 launch");
 }
 
-int ds_bf16_fault_flag(void) { return read_bf16_fault_flag(); }
+int ds_bf16_fault_flag(void) {
+  const int a = read_bf16_fault_flag(), b = read_mma_fault_flag();
+  return a < 0 || b < 0 ? -1 : (a | b);
+}
 
 void ds_bf16_set_wait_limit(long long cycles) { set_bf16_wait_cycles(cycles); }
 
@@ -489,6 +497,10 @@ ds_status ds_conv2d_shift_backward_x(const int32_t* dy, const ds_weights* w_bwd,
     r = cuda_check(cudaMemsetAsync(dx, 0, (size_t)xb, st), "dx reset");
     if (r != DS_OK) return r;
   }
+  auto launch_phases = [&](const GemmParams* ps, int n) {
+    if (!(flags & DS_CONV_IM2COL) && shift_mma_preferred(ps, n, true)) return launch_shift_mma(ps, n, true, st);
+    return launch_conv2d_shift_phases(ps, n, st);
+  };
   // output phase (rh, rw): dX rows rh, rh + sh, ...; they receive the taps r = a + sh t with
   // a = (rh + pad_h) mod sh, reading gradient row i' + c_h - t (i = sh i' + rh, c_h = (rh + pad_h - a) / sh):
   // a stride-1 correlation of dY with the phase's Th x Tw sub-kernel and padding Th - 1 - c_h
@@ -533,7 +545,7 @@ ds_status ds_conv2d_shift_backward_x(const int32_t* dy, const ds_weights* w_bwd,
       } else {
         gemm_phases[n_gemm++] = p;
         if (n_gemm == kMaxGemmPhases) {
-          r = cuda_check(launch_conv2d_shift_phases(gemm_phases, n_gemm, st),
+          r = cuda_check(launch_phases(gemm_phases, n_gemm),
                          "conv2d_shift_backward_x (implicit GEMM) launch");
           if (r != DS_OK) return r;
           n_gemm = 0;
@@ -541,7 +553,7 @@ ds_status ds_conv2d_shift_backward_x(const int32_t* dy, const ds_weights* w_bwd,
       }
     }
   if (n_gemm > 0) {
-    r = cuda_check(launch_conv2d_shift_phases(gemm_phases, n_gemm, st),
+    r = cuda_check(launch_phases(gemm_phases, n_gemm),
                    "conv2d_shift_backward_x (implicit GEMM) launch");
     if (r != DS_OK) return r;
   }
@@ -663,6 +675,8 @@ ds_status ds_conv2d_shift(const int32_t* x, const ds_weights* w, const int32_t* 
   r = prepare_amax(x, xb / (int64_t)sizeof(int32_t), flags, amax_io, st, p);
   if (r != DS_OK) return r;
   if (!(flags & DS_CONV_IM2COL)) {
+    if (shift_mma_preferred(&p, 1, true))
+      return cuda_check(launch_shift_mma(&p, 1, true, st), "conv2d_shift (tensor core) launch");
     if (conv_pointwise_supported(p))
       return cuda_check(launch_conv2d_pointwise(p, st), "conv2d_shift (pointwise) launch");
     if (conv_direct_supported(p)) return cuda_check(launch_conv2d_direct(p, st), "conv2d_shift (direct) launch");

@@ -133,6 +133,10 @@ cudaError_t launch_conv2d_shift_phases(const GemmParams* ps, int n, cudaStream_t
 // Defined in conv_narrow.cu: stride-1 ConvShift with at most 8 output columns and at most 4 taps per row.
 bool conv_narrow_supported(const GemmParams& p);
 cudaError_t launch_conv_narrow(const GemmParams& p, cudaStream_t st);
+// Defined in shift_mma.cu: exact shift sums on the tensor cores, up to kMaxGemmPhases GEMMs per launch.
+bool shift_mma_preferred(const GemmParams* ps, int n, bool conv);
+cudaError_t launch_shift_mma(const GemmParams* ps, int n, bool conv, cudaStream_t st);
+int read_mma_fault_flag();
 // Launchers (defined in shift_gemm.cu).
 cudaError_t launch_linear_shift(const GemmParams& p, cudaStream_t st);
 // Defined in linear_cluster.cu (small batches: the reduction split over a thread-block cluster).
