@@ -41,7 +41,11 @@
 // CTA: 128 rows (tensor-memory lanes) x N columns; a pair of CTAs shares a tile
 // of 256 rows, each decoding half of its weights (cta_group::2), since a tile's
 // weight bytes are written to and read from shared memory once per 128 or 256
-// rows.  25 warps:
+// rows.  25 warps, with x as operand A:
+// FC layers of up to 128 rows swap the operands' roles: the lanes are 128 weight
+// columns, decoded into tensor memory, and N = 64 rows of x are expanded into
+// shared memory, so that no lane is idle and a code is decoded once per 64 rows
+// (VGG16 FC1 at batch 64: 0.361 ms with rows as lanes, 0.206 ms so).
 //   warps 0-11   operand A, three groups of four: a thread gathers 16 values of
 //                its row, expands them and writes them to tensor memory
 //   warps 12-15  epilogue: accumulators to integer sums in shared memory, then
@@ -96,7 +100,7 @@ constexpr int kAccStride = kRows + 1;  // words between a column's sums and the 
 constexpr int kXStride = 20;    // words per staged row of 16 values: 16-byte reads of 8 rows hit all banks
 
 // Tensor-memory columns: accumulators L and H (two pairs when N = 64), then
-// three operand slots of 64 columns and two buffers of 8 + 8 digit columns.
+// three operand slots of 64 columns and two buffers of 3 x 8 digit columns.
 constexpr uint32_t kTmemSlots = 256, kTmemDigits = kTmemSlots + 64 * kSlots, kTmemCols = 512;
 
 // Column-tile flags.
@@ -106,7 +110,7 @@ constexpr uint32_t kBounded = 2;  // the columns' weights bound L and H over the
 struct PhaseInfo {
   FastDiv ohw, ow, ct;   // OH * OW, OW, column tiles
   int tile_end;          // tiles of the phases up to and including this one
-  int col_tiles, flag_off;
+  int col_tiles, flag_off, flag_tiles;
 };
 
 struct MmaSet {
@@ -160,7 +164,7 @@ __device__ __forceinline__ bool wait(uint64_t* bar, uint32_t parity, volatile in
 
 // The walk over a CTA's tiles, and in each tile over its segments (column half,
 // run, digit) and the 32-index chunks of a segment.  Every role walks alike.
-template <int GROUP>
+template <int GROUP, bool SWAP>
 struct Walk {
   const MmaSet& S;
   const uint8_t* flags;
@@ -189,7 +193,7 @@ struct Walk {
     const int local = t - (ph > 0 ? S.info[ph - 1].tile_end : 0);
     rt = fdiv(local, S.info[ph].ct);
     ct = local - rt * S.info[ph].col_tiles;
-    fl = flags[S.info[ph].flag_off + ct];
+    fl = flags[S.info[ph].flag_off + (SWAP ? rt : ct)];
     const int n = (int)S.p[ph].n_chunks;
     cb = (int)((int64_t)n * rank / S.splits);
     ce = (int)((int64_t)n * (rank + 1) / S.splits);
@@ -205,6 +209,10 @@ struct Walk {
   }
   __device__ __forceinline__ bool first_segment() const { return run == 0 && d == 0; }
   __device__ __forceinline__ bool last_segment() const { return run == runs - 1 && d == digits - 1; }
+  // Whether the last segment of the CTA's last tile (of its second half, if 64-bit) is being walked.
+  __device__ __forceinline__ bool at_end() const {
+    return last_segment() && t + t_step >= n_tiles && ((fl & kInt32) || half == 1);
+  }
   // The place in the walk, kept in shared memory between a producer warp's
   // segments (its registers are needed in between); every lane has the same.
   static constexpr int kWords = 14;
@@ -236,8 +244,8 @@ struct Walk {
   }
 };
 
-template <int GROUP>
-__device__ __forceinline__ bool next_segment_or_tile(Walk<GROUP>& w) {
+template <int GROUP, bool SWAP>
+__device__ __forceinline__ bool next_segment_or_tile(Walk<GROUP, SWAP>& w) {
   if (w.next_segment()) return true;
   if (!w.valid()) return false;
   w.start_tile();
@@ -375,40 +383,81 @@ __device__ __forceinline__ int64_t col_stride(const GemmParams& P) {
 }
 
 // The tensor operations of ring slot SLOT into accumulator pair BUF, and with
-// the second half of a chunk those of its digits.  Every operand address is a
-// constant or a base from the kernel's parameters, so the operations issue from
-// uniform registers, back to back.
-// Slot it of the CTA's sequence; go_on: 0 until the segment's first digits have
-// been issued (L's first operation is that of its first slot).
-template <int N, bool PAIR, int SLOT, int BUF>
-__device__ __forceinline__ void issue_slot(uint64_t b0, uint64_t d0, uint32_t it, uint32_t go_on, bool bounded,
+// the second half of a chunk those of its digits (buffer dbuf).  Every operand
+// address is a constant or a base from the kernel's parameters, so the
+// operations issue from uniform registers.  first: 0 for the segment's first chunk,
+// whose operations overwrite the accumulators.
+template <int N, bool PAIR, bool SWAP, int SLOT, int BUF, bool DIGITS>
+__device__ __forceinline__ void issue_slot(uint64_t b0, uint64_t d0, bool dbuf, uint32_t first, bool bounded,
                                            uint64_t* empty, uint32_t pair_mask) {
   using L = Layout<N, PAIR>;
-  constexpr uint32_t idesc = (1u << 4) | (0u << 7) | (1u << 10) | ((uint32_t)(N >> 3) << 17) |
-                             ((uint32_t)(kRows * (PAIR ? 2 : 1) >> 4) << 24);
+  // x is e4m3 (0), the weights e5m2 (1)
+  constexpr uint32_t idesc = (1u << 4) | ((SWAP ? 1u : 0u) << 7) | ((SWAP ? 0u : 1u) << 10) |
+                             ((uint32_t)(N >> 3) << 17) | ((uint32_t)(kRows * (PAIR ? 2 : 1) >> 4) << 24);
   constexpr uint32_t acc = BUF * 2 * N, a = kTmemSlots + 64 * SLOT;
-  const uint32_t first = (it & 1u) | go_on;
 #pragma unroll
   for (int j = 0; j < kSlotK / 2; ++j)
     tc::mma_f8_ts<PAIR>(acc, a + 8 * j, b0 + (uint64_t)((SLOT * L::slot_bytes >> 4) + 2 * j * L::NL), idesc,
-                        j == 0 ? first : 1u);
-  auto digit = [&](uint32_t ad, uint64_t dd) {
-    tc::mma_f8_ts<PAIR>(acc + N, ad, dd, idesc, go_on);
-    if (!bounded) {
-      tc::mma_f8_ts<PAIR>(acc, ad, dd + (uint64_t)(L::digit_bytes >> 4), idesc, 1u);
-      tc::mma_f8_ts<PAIR>(acc + N, ad + 8, dd + (uint64_t)(2 * L::digit_bytes >> 4), idesc, 1u);
-    }
-  };
-  if (it & 1u) {
-    if (it & 2u)
-      digit(kTmemDigits + 16, d0 + (uint64_t)(3 * L::digit_bytes >> 4));
+                        j == 0 && !DIGITS ? first : 1u);
+  if constexpr (DIGITS) {
+    auto digit = [&](uint32_t ad, uint64_t dd) {
+      tc::mma_f8_ts<PAIR>(acc + N, ad, dd, idesc, first);
+      if (!bounded) {
+        // x digits with the lo weights into L, x nibbles with the n3 weights into H
+        constexpr uint64_t step = L::digit_bytes >> 4;
+        tc::mma_f8_ts<PAIR>(acc, ad + (SWAP ? 8 : 0), dd + (SWAP ? 0 : step), idesc, 1u);
+        tc::mma_f8_ts<PAIR>(acc + N, ad + (SWAP ? 16 : 8), dd + (SWAP ? step : 2 * step), idesc, 1u);
+      }
+    };
+    if (dbuf)
+      digit(kTmemDigits + 24, d0 + (uint64_t)(3 * L::digit_bytes >> 4));
     else
       digit(kTmemDigits, d0);
   }
   tc::commit<PAIR>(empty + SLOT, pair_mask);
 }
 
-template <int N, bool PAIR, bool CONV, bool VEC>
+// A segment's n chunks, from ring slot 2 pos mod 3 on (pos = chunks so far mod 3;
+// the chunk loop is unrolled over the three positions, so that every slot is a
+// constant).  ring: bit s is the parity of slot s's next use.
+template <int N, bool PAIR, bool SWAP, int BUF>
+__device__ __forceinline__ bool issue_segment(Bars* bars, uint64_t b0, uint64_t d0, int n, int& pos, uint32_t& ring,
+                                              bool& dbuf, bool bounded, uint32_t pair_mask) {
+  volatile int* abort = &bars->abort;
+  uint32_t first = 0;
+  auto chunk = [&](auto p) {
+    constexpr int S0 = 2 * decltype(p)::value % 3, S1 = (S0 + 1) % 3;
+    if (!wait(&bars->full[S0], (ring >> S0) & 1u, abort)) return false;
+    tc::fence_after();
+    if (tc::elect_one()) issue_slot<N, PAIR, SWAP, S0, BUF, false>(b0, d0, dbuf, first, bounded, bars->empty, pair_mask);
+    __syncwarp();
+    if (!wait(&bars->full[S1], (ring >> S1) & 1u, abort)) return false;
+    tc::fence_after();
+    if (tc::elect_one()) issue_slot<N, PAIR, SWAP, S1, BUF, true>(b0, d0, dbuf, first, bounded, bars->empty, pair_mask);
+    __syncwarp();
+    ring ^= (1u << S0) | (1u << S1);
+    dbuf = !dbuf;
+    first = 1u;
+    return true;
+  };
+  while (true) {
+    if (pos == 0) {
+      if (!chunk(std::integral_constant<int, 0>{})) return false;
+      pos = 1;
+      if (--n == 0) return true;
+    }
+    if (pos == 1) {
+      if (!chunk(std::integral_constant<int, 1>{})) return false;
+      pos = 2;
+      if (--n == 0) return true;
+    }
+    if (!chunk(std::integral_constant<int, 2>{})) return false;
+    pos = 0;
+    if (--n == 0) return true;
+  }
+}
+
+template <int N, bool PAIR, bool CONV, bool VEC, bool SWAP>
 __global__ void __launch_bounds__(kThreads, 1) shift_mma_kernel(const __grid_constant__ MmaSet S) {
   using L = Layout<N, PAIR>;
   constexpr int NL = L::NL;            // columns whose weights this CTA decodes
@@ -491,10 +540,11 @@ __global__ void __launch_bounds__(kThreads, 1) shift_mma_kernel(const __grid_con
   const int digits = amax <= (1u << 20) ? 1 : (amax <= (1u << 24) ? 2 : (amax <= (1u << 28) ? 3 : 4));
   for (int ph = 0; ph < S.n; ++ph) {
     const GemmParams& P = S.p[ph];
-    for (int ct = warp; ct < S.info[ph].col_tiles; ct += kThreads / 32) {
+    for (int ct = warp; ct < S.info[ph].flag_tiles; ct += kThreads / 32) {
       bool wide = !have_amax || (P.flags & DS_FORCE_INT64), free = false;
-      for (int c = lane; c < N; c += 32) {
-        const int64_t col = (int64_t)ct * N + c;
+      constexpr int kTileCols = SWAP ? kRows : N;
+      for (int c = lane; c < kTileCols; c += 32) {
+        const int64_t col = (int64_t)ct * kTileCols + c;
         if (col >= P.cols) continue;
         const unsigned long long A = reinterpret_cast<const unsigned long long*>(P.blob + P.off_cola)[col];
         const unsigned long long nnz = reinterpret_cast<const uint32_t*>(P.blob + P.off_nnz)[col];
@@ -524,13 +574,13 @@ __global__ void __launch_bounds__(kThreads, 1) shift_mma_kernel(const __grid_con
       tc::mbar_arrive(bar);
   };
 
-  int* ws = reinterpret_cast<int*>(smem + kWalkOff) + warp * Walk<kGroupSize>::kWords;
-  static_assert(kWalkOff + kThreads / 32 * Walk<kGroupSize>::kWords * 4 <= kBiasOff, "one place per warp");
+  int* ws = reinterpret_cast<int*>(smem + kWalkOff) + warp * Walk<kGroupSize, SWAP>::kWords;
+  static_assert(kWalkOff + kThreads / 32 * Walk<kGroupSize, SWAP>::kWords * 4 <= kBiasOff, "one place per warp");
   const bool split = S.splits > 1;
   // a split tile of 64-bit sums goes in two passes, one per half of the columns
   int n_pass = 1;
   if (split) {
-    Walk<kGroupSize> w(S, flags, digits, 0);
+    Walk<kGroupSize, SWAP> w(S, flags, digits, 0);
     w.start_tile();
     n_pass = (w.fl & kInt32) ? 1 : 2;
   }
@@ -539,7 +589,119 @@ __global__ void __launch_bounds__(kThreads, 1) shift_mma_kernel(const __grid_con
   uint32_t ring = 0, it = 0;  // parity of the slot's use, slots so far
 
   for (int pass = 0; pass < n_pass; ++pass) {
-    if (warp < kFirstEpi) {
+    if (SWAP && warp < kFirstEpi) {
+      // ---- operand A, swapped roles: a lane is a weight column, its codes decoded into tensor memory ----
+      const int q = warp & 3;
+      slot = warp >> 2;
+      if (pass == 0) it = (uint32_t)slot;
+      const uint32_t a0 = tmem + ((uint32_t)(32 * q) << 16) + kTmemSlots + 64 * slot;
+      const uint32_t d0 = tmem + ((uint32_t)(32 * q) << 16) + kTmemDigits;
+      const uint32_t lut_a = tc::smem_u32(lut) + (lane & 7) * 16;
+      uint4* cells = reinterpret_cast<uint4*>(xrows) + tid;  // kCodeAhead slots: 16 codes, sign and non-zero plane
+      uint32_t issued = 0, used = 0, modes = 0;              // modes: bounded flags of the slots in flight
+      int rem = 0, half = 0;
+      uint32_t bounded = 0, in = 0;
+      int64_t cols = 0;
+      const unsigned char *nsrc = nullptr, *bsrc = nullptr;
+      auto seek = [&](bool first, int n) {
+        Walk<kGroupSize, SWAP> v(S, flags, digits, split ? pass : -1);
+        bool more = true;
+        if (first) {
+          v.start_tile();
+          n -= pass * 2 * (v.ce - v.cb) * digits;  // the slots of the earlier passes
+        } else {
+          v.restore(ws);
+          more = next_segment_or_tile(v);
+        }
+        while (more && n >= 2 * (v.c_end - v.chunk)) {
+          n -= 2 * (v.c_end - v.chunk);
+          more = next_segment_or_tile(v);
+        }
+        v.save(ws);
+        if (!more) return false;
+        const GemmParams& P = v.P();
+        const int64_t c = (int64_t)v.rt * kRows + 32 * q + lane;
+        cols = P.cols;
+        in = c < cols;
+        bounded = (v.fl & kBounded) ? 1u : 0u;
+        rem = 2 * (v.c_end - v.chunk) - n;
+        half = n & 1;
+        const int64_t rec = (int64_t)(v.chunk + (n >> 1)) * cols + (in ? c : 0);
+        nsrc = P.blob + P.off_nib + rec * 16;
+        bsrc = P.blob + P.off_bits + rec * 8;
+        return true;
+      };
+      bool more = seek(true, (int)it);
+      auto issue = [&]() {
+        if (more) {
+          uint4* cell = cells + (issued % kCodeAhead) * 32 * kAWarps;
+          cp_async8(cell, in ? nsrc + 8 * half : S.p[0].blob, in);
+          cp_async8(reinterpret_cast<unsigned char*>(cell) + 8, in ? bsrc : S.p[0].blob, in);
+          const uint32_t m = 1u << (issued % kCodeAhead), hm = m << 8;
+          modes = (modes & ~(m | hm)) | (bounded ? m : 0u) | (half ? hm : 0u);
+          ++issued;
+          rem -= kAGroups;
+          if (rem > 0) {
+            half += kAGroups;
+            nsrc += (half >> 1) * cols * 16;
+            bsrc += (half >> 1) * cols * 8;
+            half &= 1;
+          } else {
+            more = seek(false, -rem);
+          }
+        }
+        cp_async_commit();
+      };
+#pragma unroll 1
+      for (int i = 0; i < kCodeAhead - 1; ++i) issue();
+      for (;;) {
+        issue();
+        if (used == issued) break;
+        cp_async_wait<kCodeAhead - 1>();
+        const uint4 cell = cells[(used % kCodeAhead) * 32 * kAWarps];
+        const bool bnd = (modes >> (used % kCodeAhead)) & 1u;
+        const int h = (modes >> (8 + used % kCodeAhead)) & 1u;
+        ++used;
+        const uint32_t la = lut_a + (bnd ? 0 : kLutBytes);
+        const uint32_t sp = cell.z >> (16 * h), zp = ~cell.w >> (16 * h);
+        const uint32_t ad = d0 + 12 * (it & 2) + 4 * h;
+        if (!wait(&bars->empty[slot], ring ^ 1u, abort)) break;
+        tc::fence_after();
+#pragma unroll
+        for (int w8 = 0; w8 < 2; ++w8) {
+          const uint32_t nib = w8 ? cell.y : cell.x, sb = sp >> (8 * w8), zb = zp >> (8 * w8);
+          const uint32_t ne = ~nib & 0x0F0F0F0Fu, no = ~(nib >> 4) & 0x0F0F0F0Fu;
+          const uint32_t se = spread(sb), so = spread(sb >> 1), ze = spread(zb), zo = spread(zb >> 1);
+          const uint32_t ie = ne | (se >> 3) | (ze >> 2), io = no | (so >> 3) | (zo >> 2);
+#pragma unroll
+          for (int p = 0; p < 2; ++p) {
+            uint32_t e[16];
+#pragma unroll
+            for (int i = 0; i < 4; ++i) {
+              const uint32_t row = __byte_perm((i & 1) ? io : ie, 0, 0x4440 + 2 * p + (i >> 1));
+              asm volatile("ld.shared.v4.b32 {%0, %1, %2, %3}, [%4];"
+                           : "=r"(e[4 * i]), "=r"(e[4 * i + 1]), "=r"(e[4 * i + 2]), "=r"(e[4 * i + 3])
+                           : "r"(la + row * 128));
+            }
+            tc::st16(a0 + 32 * w8 + 16 * p, e);
+          }
+          uint32_t hi[2], lo[2], n3[2];
+          digit_weights(ne, se, ze, bnd, hi[0], lo[0], n3[0]);
+          digit_weights(no, so, zo, bnd, hi[1], lo[1], n3[1]);
+          tc::st2(ad + 2 * w8, hi[0], hi[1]);
+          if (!bnd) {
+            tc::st2(ad + 8 + 2 * w8, lo[0], lo[1]);
+            tc::st2(ad + 16 + 2 * w8, n3[0], n3[1]);
+          }
+        }
+        tc::wait_st();
+        tc::fence_before();
+        __syncwarp();
+        if (lane == 0) arrive(&bars->full[slot]);
+        it += kAGroups;
+        ring ^= 1u;
+      }
+    } else if (warp < kFirstEpi) {
       // ---- operand A: group g fills ring slot g: slots it = g, g + 3, ... of the CTA's sequence, two per chunk ----
       const int q = warp & 3;
       slot = warp >> 2;
@@ -559,7 +721,7 @@ __global__ void __launch_bounds__(kThreads, 1) shift_mma_kernel(const __grid_con
       const int32_t* tab = nullptr;
       // Moves n slots on, into later segments; false past the end of the sequence.
       auto seek = [&](bool first, int n) {
-        Walk<kGroupSize> v(S, flags, digits, split ? pass : -1);
+        Walk<kGroupSize, SWAP> v(S, flags, digits, split ? pass : -1);
         bool more = true;
         if (first) {
           v.start_tile();
@@ -676,7 +838,7 @@ __global__ void __launch_bounds__(kThreads, 1) shift_mma_kernel(const __grid_con
         }
         if (!wait(&bars->empty[slot], ring ^ 1u, abort)) break;
         tc::fence_after();
-        const uint32_t ad = d0 + 8 * (it & 2) + 4 * (it & 1);
+        const uint32_t ad = d0 + 12 * (it & 2) + 4 * (it & 1);
 #pragma unroll
         for (int hf = 0; hf < 2; ++hf) {
           uint32_t* v = CONV ? x + 8 * hf : x;
@@ -720,7 +882,7 @@ __global__ void __launch_bounds__(kThreads, 1) shift_mma_kernel(const __grid_con
     } else if (warp < kFirstB) {
       // ---- epilogue: accumulators to integer sums in shared memory (which frees them for the next
       // segment), then from there, after the tile's last segment, to the output ----
-      Walk<kGroupSize> w(S, flags, digits, split ? pass : -1);
+      Walk<kGroupSize, SWAP> w(S, flags, digits, split ? pass : -1);
       w.start_tile();
       const int q = warp & 3, rowl = 32 * q + lane;
       int32_t* bias = reinterpret_cast<int32_t*>(smem + kBiasOff) + q * N;  // this warp's copy of the tile's biases
@@ -729,7 +891,9 @@ __global__ void __launch_bounds__(kThreads, 1) shift_mma_kernel(const __grid_con
       bool more = true;
       while (more) {
         const GemmParams& P = w.P();
-        const bool i32 = (w.fl & kInt32) != 0, first = w.first_segment(), out = w.last_segment() && !split;
+        const bool i32 = (w.fl & kInt32) != 0, first = w.first_segment();
+        // split tiles' sums, and a convolution's last ones, are left to all of the CTA's warps
+        const bool out = w.last_segment() && !split && !(CONV && w.at_end());
         const int c_lo = i32 ? 0 : w.half * (N / 2), c_hi = i32 ? N : c_lo + N / 2;
         const int b = seg_no % kAccBufs, sh = 4 * w.d;
         const uint32_t acc = tmem + ((uint32_t)(32 * q) << 16) + b * 2 * N;
@@ -737,7 +901,7 @@ __global__ void __launch_bounds__(kThreads, 1) shift_mma_kernel(const __grid_con
         const int hshift = (w.fl & kBounded) ? 1 : 9;
         const float hscale = (w.fl & kBounded) ? 65536.f : 256.f;
         const int64_t col0 = (int64_t)w.ct * N;
-        if (out) {
+        if (!SWAP && out) {
           for (int c = lane; c < N; c += 32)
             bias[c] = P.bias != nullptr && col0 + c < P.cols ? __ldg(P.bias + col0 + c) : 0;
           __syncwarp();
@@ -752,14 +916,12 @@ __global__ void __launch_bounds__(kThreads, 1) shift_mma_kernel(const __grid_con
           if (i32) {
             uint32_t* a = acc32 + c0 * kAccStride;
 #pragma unroll
-            for (int j = 0; j < 16; ++j) {
-              const int lo = __float2int_rn(__uint_as_float(rl[j]) * 512.f);
-              const int hi = __float2int_rn(__uint_as_float(rh[j]) * hscale);
-              rl[j] = ((uint32_t)lo + ((uint32_t)hi << hshift)) << sh;
-            }
-            if (!first) {
+            for (int j = 0; j < 16; ++j)
+              rl[j] = (uint32_t)__float2int_rn(__uint_as_float(rl[j]) * 512.f) +
+                      ((uint32_t)__float2int_rn(__uint_as_float(rh[j]) * hscale) << hshift);
+            if (__builtin_expect(!first || sh != 0, 0)) {
 #pragma unroll
-              for (int j = 0; j < 16; ++j) rl[j] += a[j * kAccStride];
+              for (int j = 0; j < 16; ++j) rl[j] = (rl[j] << sh) + (first ? 0u : a[j * kAccStride]);
             }
 #pragma unroll
             for (int j = 0; j < 16; ++j) a[j * kAccStride] = rl[j];
@@ -782,38 +944,71 @@ __global__ void __launch_bounds__(kThreads, 1) shift_mma_kernel(const __grid_con
           const bool relu = (P.flags & DS_RELU) != 0;
           const int64_t row0 = (int64_t)w.rt * (kRows * kGroupSize) + 128 * cta + 32 * q;
           const int nc = (int)min((int64_t)(c_hi - c_lo), P.cols - col0 - c_lo);  // columns of this half that exist
-          if constexpr (CONV) {
+          if constexpr (SWAP) {
+            // lanes along the columns already; the tile's N sums of a lane are rows
+            const int64_t col = (int64_t)w.rt * kRows + rowl, r0 = (int64_t)w.ct * N + c_lo;
+            const int nr = (int)min((int64_t)(c_hi - c_lo), P.rows - r0);
+            if (col < P.cols) {
+              const int32_t bc = P.bias != nullptr ? __ldg(P.bias + col) : 0;
+              int32_t* y = P.y + r0 * P.cols + col;
+              for (int r = 0; r < nr; ++r) {
+                int32_t o = i32 ? (int32_t)(acc32[(c_lo + r) * kAccStride] + (uint32_t)bc)
+                                : sat32(acc64[r * kAccStride] + bc);
+                if (relu) o = max(o, 0);
+                amax_local = max(amax_local, uabs(o));
+                y[r * P.cols] = o;
+              }
+            }
+          } else if constexpr (CONV) {
             // lanes along the rows (pixels)
             const RowPlace rp = row_place<true>(P, S.info[w.ph], row0 + lane);
             if (rp.ok) {
               const int64_t cs = col_stride<true>(P);
-              int64_t idx = rp.y0 + (col0 + c_lo) * cs;
-              const bool resid = (P.flags & DS_RESIDUAL) != 0;
-              for (int c0 = 0; c0 < nc; c0 += 8) {
-                int32_t o[8], res[8];
-                if (resid) {
+              const int64_t idx = rp.y0 + (col0 + c_lo) * cs;
+              int32_t* y = P.y + idx;
+              const bool resid = (P.flags & DS_RESIDUAL) != 0, want_max = P.amax_out != nullptr;
+              const int32_t floor_v = relu ? 0 : INT32_MIN;
+              int c0 = 0;
+              if (i32) {
+                const int32_t* rs = P.residual + idx;
+                const uint32_t* a = acc32 + c_lo * kAccStride;
+                for (; c0 + 8 <= nc; c0 += 8) {
+                  int32_t o[8], res[8];
+                  if (resid) {
 #pragma unroll
-                  for (int j = 0; j < 8; ++j) res[j] = c0 + j < nc ? __ldg(P.residual + idx + j * cs) : 0;
-                }
+                    for (int j = 0; j < 8; ++j) res[j] = __ldg(rs + j * cs);
+                    rs += 8 * cs;
+                  }
+                  const int4 b0 = *reinterpret_cast<const int4*>(bias + c_lo + c0);
+                  const int4 b1 = *reinterpret_cast<const int4*>(bias + c_lo + c0 + 4);
+                  const int32_t bj[8] = {b0.x, b0.y, b0.z, b0.w, b1.x, b1.y, b1.z, b1.w};
 #pragma unroll
-                for (int j = 0; j < 8; ++j) {
-                  const int c = c0 + j;
-                  o[j] = i32 ? (int32_t)(acc32[(c_lo + c) * kAccStride] + (uint32_t)bias[c_lo + c])
-                             : sat32(acc64[c * kAccStride] + bias[c_lo + c]);
-                }
-                if (resid) {
+                  for (int j = 0; j < 8; ++j) o[j] = (int32_t)(a[j * kAccStride] + (uint32_t)bj[j]);
+                  a += 8 * kAccStride;
+                  if (resid) {
 #pragma unroll
-                  for (int j = 0; j < 8; ++j) o[j] = add_sat(o[j], res[j]);
-                }
+                    for (int j = 0; j < 8; ++j) o[j] = add_sat(o[j], res[j]);
+                  }
 #pragma unroll
-                for (int j = 0; j < 8; ++j) {
-                  if (relu) o[j] = max(o[j], 0);
-                  if (c0 + j < nc) {
-                    amax_local = max(amax_local, uabs(o[j]));
-                    P.y[idx + j * cs] = o[j];
+                  for (int j = 0; j < 8; ++j) {
+                    o[j] = max(o[j], floor_v);
+                    y[j * cs] = o[j];
+                  }
+                  y += 8 * cs;
+                  if (want_max) {
+#pragma unroll
+                    for (int j = 0; j < 8; ++j) amax_local = max(amax_local, uabs(o[j]));
                   }
                 }
-                idx += 8 * cs;
+              }
+              for (; c0 < nc; ++c0) {  // the columns' remainder, and 64-bit sums
+                int32_t o = i32 ? (int32_t)(acc32[(c_lo + c0) * kAccStride] + (uint32_t)bias[c_lo + c0])
+                                : sat32(acc64[c0 * kAccStride] + bias[c_lo + c0]);
+                if (resid) o = add_sat(o, __ldg(P.residual + idx + c0 * cs));
+                o = max(o, floor_v);
+                amax_local = max(amax_local, uabs(o));
+                *y = o;
+                y += cs;
               }
             }
           } else {
@@ -844,6 +1039,124 @@ __global__ void __launch_bounds__(kThreads, 1) shift_mma_kernel(const __grid_con
         ++seg_no;
         more = next_segment_or_tile(w);
       }
+    } else if (SWAP && warp < kMmaWarp) {
+      // ---- operand B, swapped roles: two groups of four warps; a thread expands 8 values of one row of x ----
+      const int tb = (warp - kFirstB) % kBSlotWarps * 32 + lane, g = (warp - kFirstB) / kBSlotWarps;
+      const int n = tb % N, kw = tb / N;  // row of the tile, which 8 of the slot's 16 indices
+      static_assert(!SWAP || N == 64, "128 threads: 64 rows x 16 indices");
+      const uint32_t dst0 = tc::smem_u32(bslots) + n * 16 + kw * 8 * N * 16;
+      const uint32_t dig0 = tc::smem_u32(bdigits) + n * 16 + kw * 8 + g * N * 16;
+      if (pass == 0) {
+        it = (uint32_t)g;
+        slot = g;
+      }
+      // kCodeAhead slots of 8 values, in flight to this thread's own words
+      int4* cells = reinterpret_cast<int4*>(xrows + kCodeAhead * kAWarps * 32 * 16) + ((warp - kFirstB) * 32 + lane);
+      uint32_t issued = 0, used = 0, modes = 0;  // modes: a byte per slot in flight: bounded flag, digit
+      int rem = 0, left = 0;
+      uint32_t mode = 0;
+      const int32_t* src = nullptr;
+      bool in = false;
+      auto seek = [&](bool first, int m) {
+        Walk<kGroupSize, SWAP> v(S, flags, digits, split ? pass : -1);
+        bool more = true;
+        if (first) {
+          v.start_tile();
+          m -= pass * 2 * (v.ce - v.cb) * digits;  // the slots of the earlier passes
+        } else {
+          v.restore(ws);
+          more = next_segment_or_tile(v);
+        }
+        while (more && m >= 2 * (v.c_end - v.chunk)) {
+          m -= 2 * (v.c_end - v.chunk);
+          more = next_segment_or_tile(v);
+        }
+        v.save(ws);
+        if (!more) return false;
+        const GemmParams& P = v.P();
+        const int64_t row = (int64_t)v.ct * N + n, k0 = (int64_t)v.chunk * kChunk + m * kSlotK + 8 * kw;
+        in = row < P.rows;
+        src = P.x + (in ? row : 0) * P.kred + k0;
+        left = (int)(P.kred - k0);
+        rem = 2 * (v.c_end - v.chunk) - m;
+        mode = ((v.fl & kBounded) ? 1u : 0u) | ((uint32_t)v.d << 1);
+        return true;
+      };
+      bool more = seek(true, (int)it);
+      auto issue = [&]() {
+        if (more) {
+          int4* cell = cells + (issued % kCodeAhead) * 64 * kBWarps;  // two halves of 4 values, 32 kBWarps apart
+          if constexpr (VEC) {
+#pragma unroll
+            for (int i = 0; i < 2; ++i) {
+              const bool ok = in && 4 * i < left;
+              cp_async16(cell + i * 32 * kBWarps, ok ? src + 4 * i : S.p[0].x, ok);
+            }
+          } else {
+#pragma unroll
+            for (int i = 0; i < 8; ++i) {
+              const bool ok = in && i < left;
+              cp_async4(reinterpret_cast<int32_t*>(cell + (i >> 2) * 32 * kBWarps) + (i & 3), ok ? src + i : S.p[0].x, ok);
+            }
+          }
+          const int at = 8 * (int)(issued % kCodeAhead);
+          modes = (modes & ~(0xFFu << at)) | (mode << at);
+          ++issued;
+          rem -= 2;
+          if (rem > 0) {
+            src += kChunk;
+            left -= kChunk;
+          } else {
+            more = seek(false, -rem);
+          }
+        }
+        cp_async_commit();
+      };
+#pragma unroll 1
+      for (int i = 0; i < kCodeAhead - 1; ++i) issue();
+      for (;;) {
+        issue();
+        if (used == issued) break;
+        cp_async_wait<kCodeAhead - 1>();
+        const int4* cell = cells + (used % kCodeAhead) * 64 * kBWarps;
+        const int4 v0 = cell[0], v1 = cell[32 * kBWarps];
+        const uint32_t now = (modes >> (8 * (used % kCodeAhead))) & 0xFFu;
+        ++used;
+        uint32_t v[8] = {(uint32_t)v0.x, (uint32_t)v0.y, (uint32_t)v0.z, (uint32_t)v0.w,
+                         (uint32_t)v1.x, (uint32_t)v1.y, (uint32_t)v1.z, (uint32_t)v1.w};
+        if (__builtin_expect(digits > 1, 0)) {
+#pragma unroll
+          for (int i = 0; i < 8; ++i) v[i] = pick_digit(v[i], (int)(now >> 1), digits);
+        }
+        if (!wait(&bars->empty[slot], ring ^ 1u, abort)) break;
+        const uint32_t dst = dst0 + slot * L::slot_bytes;
+#pragma unroll
+        for (int i = 0; i < 8; ++i) {
+          uint32_t e[4];
+          expand_x(v[i], e);
+          asm volatile("st.shared.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(dst + i * N * 16), "r"(e[0]), "r"(e[1]),
+                       "r"(e[2]), "r"(e[3])
+                       : "memory");
+        }
+        // [buffer][digits, nibbles 3][16-index half][row][16 bytes]
+        const uint32_t dd = dig0 + ((it >> 1) & 1) * 3 * L::digit_bytes;
+        asm volatile("st.shared.v2.b32 [%0], {%1, %2};" ::"r"(dd), "r"(digit4(v[0], v[2], v[4], v[6])),
+                     "r"(digit4(v[1], v[3], v[5], v[7]))
+                     : "memory");
+        if (!(now & 1u))
+          asm volatile("st.shared.v2.b32 [%0], {%1, %2};" ::"r"(dd + L::digit_bytes), "r"(nibble4(v[0], v[2], v[4], v[6])),
+                       "r"(nibble4(v[1], v[3], v[5], v[7]))
+                       : "memory");
+        tc::fence_smem_async();
+        __syncwarp();
+        if (lane == 0) arrive(&bars->full[slot]);
+        it += 2;
+        slot += 2;
+        if (slot >= kSlots) {
+          slot -= kSlots;
+          ring ^= 1u;
+        }
+      }
     } else if (warp < kMmaWarp) {
       const int bwarp = warp - kFirstB;
       // ---- operand B: two groups of four warps take turns on the slots; a thread decodes 8 codes of one
@@ -869,7 +1182,7 @@ __global__ void __launch_bounds__(kThreads, 1) shift_mma_kernel(const __grid_con
       int64_t step = 0;
       uint32_t bounded = 0, in = 0;
       auto seek = [&](bool first, int n) {
-        Walk<kGroupSize> v(S, flags, digits, split ? pass : -1);
+        Walk<kGroupSize, SWAP> v(S, flags, digits, split ? pass : -1);
         bool more = true;
         if (first) {
           v.start_tile();
@@ -973,101 +1286,101 @@ __global__ void __launch_bounds__(kThreads, 1) shift_mma_kernel(const __grid_con
         }
       }
     } else if (cta == 0) {
-      // ---- tensor operations ----
-      {
-        Walk<kGroupSize> w(S, flags, digits, split ? pass : -1);
-        w.start_tile();
-        const uint64_t b0 = tc::plain_desc(tc::smem_u32(bslots), NL * 16, 128);
-        const uint64_t d0 = tc::plain_desc(tc::smem_u32(bdigits), NL * 16, 128);
-        bool more = true, ok = true;
-        while (more) {
-          const int b = seg_no % kAccBufs;
-          ok = wait(&bars->acc_empty[b], ((uint32_t)(seg_no / kAccBufs) & 1u) ^ 1u, abort);
-          if (!ok) break;
-          tc::fence_after();
-          const bool bounded = (w.fl & kBounded) != 0;
-          const uint32_t end = it + 2 * (uint32_t)(w.c_end - w.chunk);
-          uint32_t go_on = 0;  // 0: the segment's first operation overwrites
-          for (; it != end; ++it) {
-            ok = wait(&bars->full[slot], ring, abort);
-            if (!ok) break;
-            tc::fence_after();
-            auto issue = [&](auto buf) {
-              constexpr int BUF = decltype(buf)::value;
-              if (slot == 0)
-                issue_slot<N, PAIR, 0, BUF>(b0, d0, it, go_on, bounded, bars->empty, pair_mask);
-              else if (slot == 1)
-                issue_slot<N, PAIR, 1, BUF>(b0, d0, it, go_on, bounded, bars->empty, pair_mask);
-              else
-                issue_slot<N, PAIR, 2, BUF>(b0, d0, it, go_on, bounded, bars->empty, pair_mask);
-            };
-            if (tc::elect_one()) {
-              if (kAccBufs == 1 || b == 0)
-                issue(std::integral_constant<int, 0>{});
-              else
-                issue(std::integral_constant<int, kAccBufs - 1>{});
-            }
-            __syncwarp();
-            go_on |= it & 1u;
-            if (++slot == kSlots) {
-              slot = 0;
-              ring ^= 1u;
-            }
-          }
-          if (!ok) break;
-          if (tc::elect_one()) tc::commit<PAIR>(&bars->acc_full[b], pair_mask);
-          __syncwarp();
-          ++seg_no;
-          more = next_segment_or_tile(w);
-        }
+      // ---- tensor operations (slot: chunks so far mod 3; it: digit buffer; ring: a bit per slot) ----
+      Walk<kGroupSize, SWAP> w(S, flags, digits, split ? pass : -1);
+      w.start_tile();
+      const uint64_t b0 = tc::plain_desc(tc::smem_u32(bslots), NL * 16, 128);
+      const uint64_t d0 = tc::plain_desc(tc::smem_u32(bdigits), NL * 16, 128);
+      bool more = true, dbuf = it != 0;
+      while (more) {
+        const int b = seg_no % kAccBufs, n = w.c_end - w.chunk;
+        const bool bounded = (w.fl & kBounded) != 0;
+        if (!wait(&bars->acc_empty[b], ((uint32_t)(seg_no / kAccBufs) & 1u) ^ 1u, abort)) break;
+        tc::fence_after();
+        const bool ok = kAccBufs == 1 || b == 0
+                            ? issue_segment<N, PAIR, SWAP, 0>(bars, b0, d0, n, slot, ring, dbuf, bounded, pair_mask)
+                            : issue_segment<N, PAIR, SWAP, kAccBufs - 1>(bars, b0, d0, n, slot, ring, dbuf, bounded, pair_mask);
+        if (!ok) break;
+        if (tc::elect_one()) tc::commit<PAIR>(&bars->acc_full[b], pair_mask);
+        __syncwarp();
+        ++seg_no;
+        more = next_segment_or_tile(w);
       }
-      __syncwarp();
+      it = dbuf;
     }
 
-    if (split) {
-      // the ranks' partial tiles are in their shared memory: each rank finishes its share of the columns
-      cg::cluster_group cl = cg::this_cluster();
-      tc::fence_before();
+    // The sums left in shared memory (a split tile's partial sums, one set per
+    // rank of the cluster, or a convolution's last tile of the CTA): all warps
+    // finish them, each rank its share of the columns.
+    cg::cluster_group cl = cg::this_cluster();
+    tc::fence_before();
+    if (split)
       cl.sync();
-      tc::fence_after();
-      Walk<kGroupSize> v(S, flags, digits, pass);
+    else
+      __syncthreads();
+    tc::fence_after();
+    if (CONV || split) {
+      Walk<kGroupSize, SWAP> v(S, flags, digits, split ? pass : -1);
+      while (v.t + v.t_step < v.n_tiles) v.t += v.t_step;
       v.start_tile();
       const GemmParams& P = v.P();
       const bool i32 = (v.fl & kInt32) != 0;
-      const int per = (i32 ? N : N / 2) / S.splits;
-      const int64_t cs = col_stride<CONV>(P);
-      const bool relu = (P.flags & DS_RELU) != 0;
+      const int per = (i32 ? N : N / 2) / S.splits, c_first = v.rank * per;
+      // the tile's accumulator columns are output columns, or rows with swapped roles
+      const int64_t col0 = (int64_t)v.ct * N + (i32 ? 0 : (split ? pass : 1) * (N / 2)) + c_first;
+      const int64_t row0 = (int64_t)v.rt * (kRows * kGroupSize) + 128 * cta;
+      const int nc = (int)min((int64_t)per, (SWAP ? P.rows : P.cols) - col0);
+      const int32_t floor_v = (P.flags & DS_RELU) ? 0 : INT32_MIN;
       uint32_t amax_local = 0;
-      for (int e = tid; e < per * kRows; e += kThreads) {
-        const int c = v.rank * per + e / kRows, row = e % kRows;
-        const int64_t col = (int64_t)v.ct * N + (i32 ? 0 : pass * (N / 2)) + c;
-        const RowPlace rp = row_place<CONV>(P, S.info[v.ph], (int64_t)v.rt * (kRows * kGroupSize) + 128 * cta + row);
-        if (!rp.ok || col >= P.cols) continue;
-        long long sum = P.bias != nullptr ? __ldg(P.bias + col) : 0;
+      auto finish = [&](int c, int row, int64_t idx) {
+        long long sum = P.bias != nullptr ? __ldg(P.bias + (SWAP ? row0 + row : col0 + c)) : 0;
+        const int at = (c_first + c) * kAccStride + row;
         if (i32) {
-          uint32_t s32 = 0;
-          for (int q = 0; q < S.splits; ++q)
-            s32 += *cl.map_shared_rank(reinterpret_cast<uint32_t*>(accs) + c * kAccStride + row, q * kGroupSize + cta);
+          uint32_t s32 = reinterpret_cast<uint32_t*>(accs)[at];
+          if (split) {
+            s32 = 0;
+            for (int q = 0; q < S.splits; ++q)
+              s32 += *cl.map_shared_rank(reinterpret_cast<uint32_t*>(accs) + at, q * kGroupSize + cta);
+          }
           sum = (int32_t)(s32 + (uint32_t)sum);
-        } else {
+        } else if (split) {
           for (int q = 0; q < S.splits; ++q)
-            sum += *cl.map_shared_rank(reinterpret_cast<long long*>(accs) + c * kAccStride + row, q * kGroupSize + cta);
+            sum += *cl.map_shared_rank(reinterpret_cast<long long*>(accs) + at, q * kGroupSize + cta);
           sum = sat32(sum);
+        } else {
+          sum = sat32(sum + reinterpret_cast<long long*>(accs)[at]);
         }
         int32_t o = (int32_t)sum;
-        const int64_t idx = rp.y0 + col * cs;
         if (CONV && (P.flags & DS_RESIDUAL)) o = add_sat(o, __ldg(P.residual + idx));
-        if (relu) o = max(o, 0);
+        o = max(o, floor_v);
         amax_local = max(amax_local, uabs(o));
         P.y[idx] = o;
+      };
+      if constexpr (SWAP) {  // a thread keeps its output column
+        constexpr int kRowGroups = kThreads / kRows;
+        const int64_t col = row0 + tid % kRows;
+        if (col < P.cols && tid < kRowGroups * kRows)
+          for (int r = tid / kRows; r < nc; r += kRowGroups) finish(r, tid % kRows, (col0 + r) * P.cols + col);
+      } else if constexpr (CONV) {  // a thread keeps its row
+        constexpr int kColGroups = kThreads / kRows;
+        const int64_t cs = col_stride<true>(P);
+        const RowPlace rp = row_place<true>(P, S.info[v.ph], row0 + tid % kRows);
+        if (rp.ok && tid < kColGroups * kRows) {
+#pragma unroll 4
+          for (int c = tid / kRows; c < nc; c += kColGroups) finish(c, tid % kRows, rp.y0 + (col0 + c) * cs);
+        }
+      } else {  // a warp takes rows, its lanes the columns
+        const int nr = (int)min((int64_t)kRows, P.rows - row0);
+        for (int row = warp; row < nr; row += kThreads / 32)
+          for (int c = lane; c < nc; c += 32) finish(c, row, (row0 + row) * P.cols + col0 + c);
       }
       __syncwarp();
       if (P.amax_out != nullptr) {
         amax_local = __reduce_max_sync(0xffffffffu, amax_local);
         if (lane == 0 && amax_local) atomicMax(P.amax_out, amax_local);
       }
-      cl.sync();  // the peers' reads end before this shared memory changes
     }
+    if (split) cl.sync();  // the peers' reads end before this shared memory changes
   }
 
   // every tensor operation has completed, in both CTAs of a pair, before tensor memory is freed
@@ -1087,13 +1400,13 @@ __global__ void __launch_bounds__(kThreads, 1) shift_mma_kernel(const __grid_con
   }
 }
 
-template <int N, bool PAIR, bool CONV, bool VEC>
+template <int N, bool PAIR, bool CONV, bool VEC, bool SWAP>
 bool set_attributes() {
   // once per process, thread-safe (see conv_direct.cu)
   static const bool ok = [] {
-    const bool r = cudaFuncSetAttribute(shift_mma_kernel<N, PAIR, CONV, VEC>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+    const bool r = cudaFuncSetAttribute(shift_mma_kernel<N, PAIR, CONV, VEC, SWAP>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                         227 * 1024) == cudaSuccess &&
-                   cudaFuncSetAttribute(shift_mma_kernel<N, PAIR, CONV, VEC>, cudaFuncAttributeNonPortableClusterSizeAllowed,
+                   cudaFuncSetAttribute(shift_mma_kernel<N, PAIR, CONV, VEC, SWAP>, cudaFuncAttributeNonPortableClusterSizeAllowed,
                                         1) == cudaSuccess;
     if (!r) (void)cudaGetLastError();
     return r;
@@ -1102,7 +1415,7 @@ bool set_attributes() {
 }
 
 // How many clusters of cs CTAs the device holds at once (one CTA per SM), read once per size.
-template <int N, bool PAIR, bool CONV, bool VEC>
+template <int N, bool PAIR, bool CONV, bool VEC, bool SWAP>
 int max_clusters(int cs) {
   static int cache[kMaxCluster + 1] = {};
   static std::mutex mu;
@@ -1120,7 +1433,7 @@ int max_clusters(int cs) {
     cfg.attrs = &attr;
     cfg.numAttrs = 1;
     int n = 0;
-    if (cudaOccupancyMaxActiveClusters(&n, shift_mma_kernel<N, PAIR, CONV, VEC>, &cfg) != cudaSuccess) {
+    if (cudaOccupancyMaxActiveClusters(&n, shift_mma_kernel<N, PAIR, CONV, VEC, SWAP>, &cfg) != cudaSuccess) {
       (void)cudaGetLastError();
       n = 0;
     }
@@ -1129,9 +1442,9 @@ int max_clusters(int cs) {
   return cache[cs] > 0 ? cache[cs] : 0;
 }
 
-template <int N, bool PAIR, bool CONV, bool VEC>
+template <int N, bool PAIR, bool CONV, bool VEC, bool SWAP>
 cudaError_t launch_n(MmaSet& S, int tiles, cudaStream_t st) {
-  if (!set_attributes<N, PAIR, CONV, VEC>()) return cudaErrorInvalidValue;
+  if (!set_attributes<N, PAIR, CONV, VEC, SWAP>()) return cudaErrorInvalidValue;
   const int sms = sm_count();
   if (sms <= 0) return cudaErrorNoDevice;
   int nch = INT32_MAX;
@@ -1139,12 +1452,12 @@ cudaError_t launch_n(MmaSet& S, int tiles, cudaStream_t st) {
   // split sizes 1, 2, 4, .. (clusters of at most 16 CTAs): the least waves x
   // chunks of a rank, plus a fixed cost of the cluster reduction
   constexpr int group = PAIR ? 2 : 1;
-  const int units = PAIR ? std::max(1, max_clusters<N, PAIR, CONV, VEC>(group)) : sms;
+  const int units = PAIR ? std::max(1, max_clusters<N, PAIR, CONV, VEC, SWAP>(group)) : sms;
   S.splits = 1;
   int64_t best = (int64_t)((tiles + units - 1) / units) * (nch + 4);
   if (tiles < units)
     for (int cs = 2; cs * group <= kMaxCluster && 2 * cs <= nch; cs *= 2) {
-      const int n = max_clusters<N, PAIR, CONV, VEC>(cs * group);
+      const int n = max_clusters<N, PAIR, CONV, VEC, SWAP>(cs * group);
       if (n <= 0) continue;
       const int64_t cost = (int64_t)((tiles + n - 1) / n) * ((nch + cs - 1) / cs + 6);
       if (cost < best) {
@@ -1165,10 +1478,10 @@ cudaError_t launch_n(MmaSet& S, int tiles, cudaStream_t st) {
   attr.val.clusterDim.z = 1;
   cfg.attrs = &attr;
   cfg.numAttrs = S.splits * group > 1 ? 1 : 0;
-  return cudaLaunchKernelEx(&cfg, shift_mma_kernel<N, PAIR, CONV, VEC>, S);
+  return cudaLaunchKernelEx(&cfg, shift_mma_kernel<N, PAIR, CONV, VEC, SWAP>, S);
 }
 
-template <int N, bool PAIR>
+template <int N, bool PAIR, bool SWAP = false>
 cudaError_t launch_set(const GemmParams* ps, int n, bool conv, cudaStream_t st) {
   MmaSet S{};
   S.n = n;
@@ -1180,20 +1493,25 @@ cudaError_t launch_set(const GemmParams* ps, int n, bool conv, cudaStream_t st) 
     const GemmParams& p = ps[i];
     S.p[i] = p;
     PhaseInfo& f = S.info[i];
-    f.col_tiles = (int)((p.cols + N - 1) / N);
+    f.col_tiles = (int)(((SWAP ? p.rows : p.cols) + N - 1) / N);
     f.ct = make_fastdiv((uint32_t)f.col_tiles);
     f.ohw = make_fastdiv(conv ? (uint32_t)(p.OH * p.OW) : 1u);
     f.ow = make_fastdiv(conv ? (uint32_t)p.OW : 1u);
-    f.flag_off = flag_off;
-    flag_off += f.col_tiles;
     constexpr int rows = kRows * (PAIR ? 2 : 1);
-    tiles += (p.rows + rows - 1) / rows * f.col_tiles;
+    const int64_t row_tiles = ((SWAP ? p.cols : p.rows) + rows - 1) / rows;
+    f.flag_off = flag_off;
+    f.flag_tiles = SWAP ? (int)row_tiles : f.col_tiles;
+    flag_off += f.flag_tiles;
+    tiles += row_tiles * f.col_tiles;
     f.tile_end = (int)tiles;
     if (conv) S.table_entries = std::max(S.table_entries, (p.R * p.S + kSlotK + 3) / 4 * 4);
     vec = vec && p.kred % 4 == 0;
   }
-  if (conv) return launch_n<N, PAIR, true, false>(S, (int)tiles, st);
-  return vec ? launch_n<N, PAIR, false, true>(S, (int)tiles, st) : launch_n<N, PAIR, false, false>(S, (int)tiles, st);
+  if constexpr (!SWAP) {
+    if (conv) return launch_n<N, PAIR, true, false, false>(S, (int)tiles, st);
+  }
+  return vec ? launch_n<N, PAIR, false, true, SWAP>(S, (int)tiles, st)
+             : launch_n<N, PAIR, false, false, SWAP>(S, (int)tiles, st);
 }
 
 }  // namespace
@@ -1201,16 +1519,20 @@ cudaError_t launch_set(const GemmParams* ps, int n, bool conv, cudaStream_t st) 
 // Rules of use, measured against the CUDA-core kernels.  A tile's fixed cost (its
 // epilogue, the ring's fill) is that of about 100 reduction indices: 1x1 layers of
 // 64 channels and 3x3 layers of 3 ran at 0.5-0.6 of the CUDA-core kernels' speed,
-// the 147 indices of a 7x7 layer of 3 channels at 1.2.  FC of 32 rows of 25088
-// indices ran at 0.92, 64 rows at 1.6; 64 rows of 784 indices at 1.0, 256 rows of
-// 2048 at 1.6.
+// the 147 indices of a 7x7 layer of 3 channels at 1.2.  A launch's fixed cost (table,
+// tensor memory, cluster) is 3-4 us: FC of 64 x 2048 x 1000 (2^27 terms) ran at 1.2,
+// of 16 x 2048 x 1000 at 0.9; a convolution of 2^27 terms at 1.1.  Up to 8 rows an FC
+// layer is bound by its codes, which the cluster kernel reads once (8 x 25088 x
+// 4096: 0.94; 16 rows: 1.8).
 bool shift_mma_preferred(const GemmParams* ps, int n, bool conv) {
   if (n < 1 || n > kMaxGemmPhases) return false;
   int64_t tiles = 0, col_tiles = 0;
+  double terms = 0.0;
   for (int i = 0; i < n; ++i) {
     const GemmParams& p = ps[i];
     if (p.rows > INT32_MAX - kRows || p.n_chunks > INT32_MAX / kChunk) return false;
-    if (conv ? p.kred < 128 || p.rows < 1024 : p.rows < 64 || (p.rows < 256 && p.kred < 2048)) return false;
+    if (conv ? p.kred < 128 || p.rows < 1024 : p.rows <= 8) return false;
+    terms += (double)p.rows * (double)p.kred * (double)p.cols;
     col_tiles += (p.cols + 63) / 64;
     tiles += (p.rows + kRows - 1) / kRows * ((p.cols + 63) / 64);
     if (conv) {
@@ -1219,6 +1541,7 @@ bool shift_mma_preferred(const GemmParams* ps, int n, bool conv) {
       if ((int64_t)(kAGroups * kSlotK + 8) * p.H * p.W + (int64_t)p.R * p.W > INT32_MAX) return false;
     }
   }
+  if (terms < (conv ? 67108864.0 : 134217728.0)) return false;
   return col_tiles <= kMaxColTiles && tiles <= INT32_MAX / kMaxCluster;
 }
 
@@ -1228,6 +1551,7 @@ cudaError_t launch_shift_mma(const GemmParams* ps, int n, bool conv, cudaStream_
     cols = std::max(cols, ps[i].cols);
     rows = std::max(rows, ps[i].rows);
   }
+  if (!conv && rows <= kRows) return launch_set<64, false, true>(ps, n, conv, st);
   if (rows <= kRows) return launch_set<64, false>(ps, n, conv, st);
   return cols <= 64 ? launch_set<64, true>(ps, n, conv, st) : launch_set<128, true>(ps, n, conv, st);
 }
