@@ -42,10 +42,6 @@
 // of 256 rows, each decoding half of its weights (cta_group::2), since a tile's
 // weight bytes are written to and read from shared memory once per 128 or 256
 // rows.  25 warps, with x as operand A:
-// FC layers of up to 128 rows swap the operands' roles: the lanes are 128 weight
-// columns, decoded into tensor memory, and N = 64 rows of x are expanded into
-// shared memory, so that no lane is idle and a code is decoded once per 64 rows
-// (VGG16 FC1 at batch 64: 0.361 ms with rows as lanes, 0.206 ms so).
 //   warps 0-11   operand A, three groups of four: a thread gathers 16 values of
 //                its row, expands them and writes them to tensor memory
 //   warps 12-15  epilogue: accumulators to integer sums in shared memory, then
@@ -53,6 +49,10 @@
 //   warps 16-23  operand B, two groups of four: decode the packed codes of a
 //                column through a table of weight bytes into shared memory
 //   warp 24      issues the tensor operations
+// FC layers of up to 128 rows swap the operands' roles: the lanes are 128 weight
+// columns, decoded into tensor memory, and N = 64 rows of x are expanded into
+// shared memory, so that no lane is idle and a code is decoded once per 64 rows
+// (VGG16 FC1 at batch 64: 0.361 ms with rows as lanes, 0.206 ms so).
 // A ring of three slots of 16 reduction indices connects them; CTAs are
 // persistent over tiles and the ring runs on across them.  A grid that leaves
 // SMs idle splits the reduction over the CTAs of a cluster, which sum their
@@ -121,7 +121,7 @@ struct MmaSet {
 
 struct __align__(8) Bars {
   uint64_t full[kSlots], empty[kSlots], acc_full[2], acc_empty[2], done;
-  uint32_t tmem;
+  uint32_t tmem, amax;
   int abort;
 };
 
@@ -494,70 +494,78 @@ __global__ void __launch_bounds__(kThreads, 1) shift_mma_kernel(const __grid_con
     }
     tc::mbar_init(&bars->done, 1);
     bars->abort = 0;
+    bars->amax = 0;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
   if (warp == kMmaWarp) tc::tmem_alloc<PAIR>(&bars->tmem, kTmemCols);
-  // weight bytes by code: row sh ^ 15 | negative << 4 | zero << 5, eight copies
-  // of 16 bytes per row, so that 8 lanes reading any rows hit all banks once
-  // (the second table leaves nibble 3 out for sh < 4, see above)
-  for (int i = tid; i < 2 * 64 * 8; i += kThreads) {
-    const int row = (i >> 3) & 63, sh = 15 - (row & 15);
-    // byte q: the weight 2^(4q - sh) as e5m2
-    uint32_t e = 0x04040404u * (uint32_t)(15 - sh) + 0x30201000u;
-    if (row & 16) e |= 0x80808080u;
-    if (i >= 512 && sh < 4) e &= 0x00FFFFFFu;
-    if (row >= 32) e = 0u;
-    uint32_t w[4];
-#pragma unroll
-    for (int j = 0; j < 4; ++j) {
-      const int cut = 8 * ((sh - j + 3) >> 2);  // bits of the bytes q with 4q + j < sh
-      w[j] = cut < 32 ? e & (~0u << cut) : 0u;
-    }
-    *reinterpret_cast<uint4*>(lut + i * 16) = make_uint4(w[0], w[1], w[2], w[3]);
-  }
-  if (CONV) {
-    // taps of 16 consecutive reduction indices: element offsets, then kernel
-    // row / column bits.  Copy c = 0..3 starts at tap c, so that 16-byte reads can
-    // start anywhere; the last 32 entries are the taps of the reduction's partial
-    // last slot, its missing ones (and 16 more) marked as never valid.
-    for (int ph = 0; ph < S.n; ++ph) {
-      const GemmParams& P = S.p[ph];
-      const int rs = P.R * P.S, te = S.table_entries, tail = (int)(P.kred % kSlotK);
-      const int t0 = (int)((P.kred - tail) % rs);
-      for (int e = tid; e < 4 * te + 32; e += kThreads) {
-        const bool in_tail = e >= 4 * te;
-        const int i = in_tail ? t0 + e - 4 * te : e / te + e % te;
-        const int c = i / rs, tap = i - c * rs, r = tap / P.S, q = tap - r * P.S;
-        const bool never = in_tail && e - 4 * te >= tail;
-        int32_t* t = tables + ph * 2 * (4 * te + 32) + e;
-        t[0] = never ? 0 : c * P.H * P.W + r * P.W + q;
-        t[4 * te + 32] = never ? INT32_MIN : (int32_t)((1u << r) | (0x10000u << q));
-      }
-    }
-  }
   const bool have_amax = S.p[0].amax_in != nullptr;
   const uint32_t amax = have_amax ? *S.p[0].amax_in : 0x80000000u;
   const int digits = amax <= (1u << 20) ? 1 : (amax <= (1u << 24) ? 2 : (amax <= (1u << 28) ? 3 : 4));
-  for (int ph = 0; ph < S.n; ++ph) {
-    const GemmParams& P = S.p[ph];
-    for (int ct = warp; ct < S.info[ph].flag_tiles; ct += kThreads / 32) {
-      bool wide = !have_amax || (P.flags & DS_FORCE_INT64), free = false;
-      constexpr int kTileCols = SWAP ? kRows : N;
-      for (int c = lane; c < kTileCols; c += 32) {
-        const int64_t col = (int64_t)ct * kTileCols + c;
-        if (col >= P.cols) continue;
-        const unsigned long long A = reinterpret_cast<const unsigned long long*>(P.blob + P.off_cola)[col];
-        const unsigned long long nnz = reinterpret_cast<const uint32_t*>(P.blob + P.off_nnz)[col];
-        const unsigned long long b = P.bias ? (unsigned long long)uabs(P.bias[col]) : 0ull;
-        // 2^31 * A and every product below stay inside 64 bits for A < 2^32; a larger A fails both bounds
-        const bool huge = (A >> 32) != 0;
-        wide |= huge || ((((unsigned long long)amax * A + 32767ull) >> 15) + nnz + b > (unsigned long long)INT32_MAX);
-        const unsigned long long u = digits > 1 ? 16u : (amax + 65535u) >> 16;  // max |digit|
-        free |= huge || 2 * A > (1ull << 24) || u * A > (1ull << 24);
+  // A convolution's column flags and tables are made by different warps side by
+  // side (its launches are many and short: 1-2 us of each); FC's by all warps.
+  constexpr int kFlagWarps = CONV ? 12 : kThreads / 32, kTableWarp = CONV ? kFlagWarps : 0;
+  if (warp < kFlagWarps) {
+    for (int ph = 0; ph < S.n; ++ph) {
+      const GemmParams& P = S.p[ph];
+      for (int ct = warp; ct < S.info[ph].flag_tiles; ct += kFlagWarps) {
+        bool wide = !have_amax || (P.flags & DS_FORCE_INT64), free = false;
+        constexpr int kTileCols = SWAP ? kRows : N;
+        for (int c = lane; c < kTileCols; c += 32) {
+          const int64_t col = (int64_t)ct * kTileCols + c;
+          if (col >= P.cols) continue;
+          const unsigned long long A = reinterpret_cast<const unsigned long long*>(P.blob + P.off_cola)[col];
+          const unsigned long long nnz = reinterpret_cast<const uint32_t*>(P.blob + P.off_nnz)[col];
+          const unsigned long long b = P.bias ? (unsigned long long)uabs(P.bias[col]) : 0ull;
+          // 2^31 * A and every product below stay inside 64 bits for A < 2^32; a larger A fails both bounds
+          const bool huge = (A >> 32) != 0;
+          wide |= huge || ((((unsigned long long)amax * A + 32767ull) >> 15) + nnz + b > (unsigned long long)INT32_MAX);
+          const unsigned long long u = digits > 1 ? 16u : (amax + 65535u) >> 16;  // max |digit|
+          free |= huge || 2 * A > (1ull << 24) || u * A > (1ull << 24);
+        }
+        const uint32_t f =
+            (__any_sync(0xffffffffu, wide) ? 0u : kInt32) | (__any_sync(0xffffffffu, free) ? 0u : kBounded);
+        if (lane == 0) flags[S.info[ph].flag_off + ct] = (uint8_t)f;
       }
-      const uint32_t f =
-          (__any_sync(0xffffffffu, wide) ? 0u : kInt32) | (__any_sync(0xffffffffu, free) ? 0u : kBounded);
-      if (lane == 0) flags[S.info[ph].flag_off + ct] = (uint8_t)f;
+    }
+  }
+  if (warp >= kTableWarp) {
+    // weight bytes by code: row sh ^ 15 | negative << 4 | zero << 5, eight copies
+    // of 16 bytes per row, so that 8 lanes reading any rows hit all banks once
+    // (the second table leaves nibble 3 out for sh < 4, see above)
+    for (int i = tid - 32 * kTableWarp; i < 2 * 64 * 8; i += kThreads - 32 * kTableWarp) {
+      const int row = (i >> 3) & 63, sh = 15 - (row & 15);
+      // byte q: the weight 2^(4q - sh) as e5m2
+      uint32_t e = 0x04040404u * (uint32_t)(15 - sh) + 0x30201000u;
+      if (row & 16) e |= 0x80808080u;
+      if (i >= 512 && sh < 4) e &= 0x00FFFFFFu;
+      if (row >= 32) e = 0u;
+      uint32_t w[4];
+#pragma unroll
+      for (int j = 0; j < 4; ++j) {
+        const int cut = 8 * ((sh - j + 3) >> 2);  // bits of the bytes q with 4q + j < sh
+        w[j] = cut < 32 ? e & (~0u << cut) : 0u;
+      }
+      *reinterpret_cast<uint4*>(lut + i * 16) = make_uint4(w[0], w[1], w[2], w[3]);
+    }
+    if (CONV) {
+      // taps of 16 consecutive reduction indices: element offsets, then kernel
+      // row / column bits.  Copy c = 0..3 starts at tap c, so that 16-byte reads can
+      // start anywhere; the last 32 entries are the taps of the reduction's partial
+      // last slot, its missing ones (and 16 more) marked as never valid.
+      for (int ph = 0; ph < S.n; ++ph) {
+        const GemmParams& P = S.p[ph];
+        const int rs = P.R * P.S, te = S.table_entries, tail = (int)(P.kred % kSlotK);
+        const int t0 = (int)((P.kred - tail) % rs);
+        for (int e = tid - 32 * kTableWarp; e < 4 * te + 32; e += kThreads - 32 * kTableWarp) {
+          const bool in_tail = e >= 4 * te;
+          const int i = in_tail ? t0 + e - 4 * te : e / te + e % te;
+          const int c = i / rs, tap = i - c * rs, r = tap / P.S, q = tap - r * P.S;
+          const bool never = in_tail && e - 4 * te >= tail;
+          int32_t* t = tables + ph * 2 * (4 * te + 32) + e;
+          t[0] = never ? 0 : c * P.H * P.W + r * P.W + q;
+          t[4 * te + 32] = never ? INT32_MIN : (int32_t)((1u << r) | (0x10000u << q));
+        }
+      }
     }
   }
   tc::fence_before();
@@ -1366,8 +1374,56 @@ __global__ void __launch_bounds__(kThreads, 1) shift_mma_kernel(const __grid_con
         const int64_t cs = col_stride<true>(P);
         const RowPlace rp = row_place<true>(P, S.info[v.ph], row0 + tid % kRows);
         if (rp.ok && tid < kColGroups * kRows) {
-#pragma unroll 4
-          for (int c = tid / kRows; c < nc; c += kColGroups) finish(c, tid % kRows, rp.y0 + (col0 + c) * cs);
+          // Eight outputs of a thread at a time, their loads (bias, residual, the peers'
+          // sums) in flight together: one at a time this took 10-17 thousand clocks a tile.
+          // place(j, c, row, idx): output j's accumulator column, lane and output element; false if there is none.
+          auto finish8 = [&](auto place) {
+            int at[8];
+            int64_t idx[8];
+            int32_t o[8], res[8];
+            bool ok[8];
+#pragma unroll
+            for (int j = 0; j < 8; ++j) {
+              int c = 0, row = 0;
+              ok[j] = place(j, c, row, idx[j]);
+              at[j] = (c_first + c) * kAccStride + row;
+              o[j] = ok[j] && P.bias != nullptr ? __ldg(P.bias + col0 + c) : 0;
+              res[j] = ok[j] && (P.flags & DS_RESIDUAL) ? __ldg(P.residual + idx[j]) : 0;
+              if (!ok[j]) at[j] = 0;
+            }
+            if (i32) {
+              uint32_t* sums = reinterpret_cast<uint32_t*>(accs);
+              for (int q = 0; q < S.splits; ++q) {
+                const uint32_t* src = split ? cl.map_shared_rank(sums, q * kGroupSize + cta) : sums;
+#pragma unroll
+                for (int j = 0; j < 8; ++j) o[j] = (int32_t)((uint32_t)o[j] + src[at[j]]);
+              }
+            } else {
+              long long* sums = reinterpret_cast<long long*>(accs);
+#pragma unroll
+              for (int j = 0; j < 8; ++j) {
+                long long v = o[j];
+                for (int q = 0; q < S.splits; ++q) v += (split ? cl.map_shared_rank(sums, q * kGroupSize + cta) : sums)[at[j]];
+                o[j] = sat32(v);
+              }
+            }
+#pragma unroll
+            for (int j = 0; j < 8; ++j) {
+              if ((P.flags & DS_RESIDUAL) != 0) o[j] = add_sat(o[j], res[j]);
+              o[j] = max(o[j], floor_v);
+              if (ok[j]) {
+                amax_local = max(amax_local, uabs(o[j]));
+                P.y[idx[j]] = o[j];
+              }
+            }
+          };
+          for (int b0 = tid / kRows; b0 < nc; b0 += 8 * kColGroups)
+            finish8([&](int j, int& c, int& row, int64_t& idx) {
+              c = b0 + j * kColGroups;
+              row = tid % kRows;
+              idx = rp.y0 + (col0 + c) * cs;
+              return c < nc;
+            });
         }
       } else {  // a warp takes rows, its lanes the columns
         const int nr = (int)min((int64_t)kRows, P.rows - row0);
@@ -1375,9 +1431,9 @@ __global__ void __launch_bounds__(kThreads, 1) shift_mma_kernel(const __grid_con
           for (int c = lane; c < nc; c += 32) finish(c, row, (row0 + row) * P.cols + col0 + c);
       }
       __syncwarp();
-      if (P.amax_out != nullptr) {
+      if (P.amax_out != nullptr) {  // convolutions: one global atomic per CTA instead of one per warp
         amax_local = __reduce_max_sync(0xffffffffu, amax_local);
-        if (lane == 0 && amax_local) atomicMax(P.amax_out, amax_local);
+        if (lane == 0 && amax_local) atomicMax(CONV ? &bars->amax : P.amax_out, amax_local);
       }
     }
     if (split) cl.sync();  // the peers' reads end before this shared memory changes
@@ -1385,6 +1441,7 @@ __global__ void __launch_bounds__(kThreads, 1) shift_mma_kernel(const __grid_con
 
   // every tensor operation has completed, in both CTAs of a pair, before tensor memory is freed
   __syncthreads();
+  if (CONV && tid == 0 && bars->amax && S.p[0].amax_out != nullptr) atomicMax(S.p[0].amax_out, bars->amax);
   if (warp == kMmaWarp) {
     if (cta == 0 && tc::elect_one()) tc::commit<PAIR>(&bars->done, pair_mask);
     __syncwarp();
