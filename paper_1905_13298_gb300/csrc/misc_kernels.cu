@@ -444,6 +444,35 @@ __global__ void absmax_kernel(const int32_t* __restrict__ x, int64_t n, uint32_t
   }
 }
 
+// Up to kSmallAbsmax values: one block, which writes its maximum over the old
+// word, so that no reset goes before it.  A latency-bound call (a network's
+// classifier at batch 1 is 512 values) is three launches otherwise, of which the
+// reset's and its gap are about 2 us.
+constexpr int64_t kSmallAbsmax = 1 << 14;
+__global__ void __launch_bounds__(1024) absmax_small_kernel(const int32_t* __restrict__ x, int n, uint32_t* out) {
+  uint32_t m = 0;
+  if ((reinterpret_cast<uintptr_t>(x) & 15) == 0) {
+    const int nv = n >> 2;
+    const int4* xv = reinterpret_cast<const int4*>(x);
+#pragma unroll 4
+    for (int i = threadIdx.x; i < nv; i += 1024) {
+      const int4 v = __ldg(xv + i);
+      m = max(m, max(max(uabs(v.x), uabs(v.y)), max(uabs(v.z), uabs(v.w))));
+    }
+    for (int i = (nv << 2) + threadIdx.x; i < n; i += 1024) m = max(m, uabs(x[i]));
+  } else {
+    for (int i = threadIdx.x; i < n; i += 1024) m = max(m, uabs(x[i]));
+  }
+  __shared__ uint32_t wmax[32];
+  m = __reduce_max_sync(0xffffffffu, m);
+  if ((threadIdx.x & 31) == 0) wmax[threadIdx.x >> 5] = m;
+  __syncthreads();
+  if (threadIdx.x < 32) {
+    const uint32_t v = __reduce_max_sync(0xffffffffu, wmax[threadIdx.x]);
+    if (threadIdx.x == 0) *out = v;
+  }
+}
+
 int sm_count() {
   // read once per process (thread-safe function-local static); the library
   // serves one device per process
@@ -462,6 +491,10 @@ int sm_count() {
 cudaError_t launch_absmax(const int32_t* x, int64_t n, uint32_t* out, cudaStream_t st) {
   const int sms = sm_count();
   if (sms <= 0) return cudaErrorNoDevice;
+  if (n <= kSmallAbsmax) {
+    absmax_small_kernel<<<1, 1024, 0, st>>>(x, (int)n, out);
+    return cudaGetLastError();
+  }
   cudaError_t e = cudaMemsetAsync(out, 0, sizeof(uint32_t), st);
   if (e != cudaSuccess) return e;
   const int threads = 256;
