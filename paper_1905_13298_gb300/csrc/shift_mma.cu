@@ -85,13 +85,17 @@ constexpr int kSlotK = 16;      // reduction indices per ring slot
 constexpr int kSlots = 3;
 constexpr int kRunChunks = 120; // chunks of 32 per run of a tile with unbounded columns
 constexpr int kAGroups = 3;     // four warps each; group g fills ring slot g
-constexpr int kAWarps = 4 * kAGroups, kEpiWarps = 4, kBWarps = 8;
+constexpr int kAWarps = 4 * kAGroups, kEpiWarps = 4;
 static_assert(kAGroups == kSlots, "a group of operand-A warps per ring slot");
-// warps 0-11 operand A, 12-15 epilogue, 16-23 operand B, 24 tensor operations
-constexpr int kFirstEpi = kAWarps, kFirstB = kFirstEpi + kEpiWarps, kMmaWarp = kFirstB + kBWarps;
-constexpr int kThreads = 32 * (kMmaWarp + 1);
+// warps 0-11 operand A, 12-15 epilogue, then operand B, then the tensor operations
+constexpr int kFirstEpi = kAWarps, kFirstB = kFirstEpi + kEpiWarps;
+// Operand B: three groups of two warps, or with swapped roles two of four.  23
+// warps leave a thread 80 registers, 25 leave 72: with 72 the convolution's operand
+// A spills in its loop (a version with 270 spilled bytes ran 15-30% slower).
+__host__ __device__ constexpr int b_warps(bool swap) { return swap ? 8 : 6; }
+__host__ __device__ constexpr int cta_threads(bool swap) { return 32 * (kFirstB + b_warps(swap) + 1); }
 constexpr int kCodeAhead = 4;   // slots of a B group whose codes are in flight
-constexpr int kCodeBytes = kCodeAhead * kBWarps * 32 * 16;
+constexpr int kCodeBytes = kCodeAhead * b_warps(false) * 32 * 16;
 constexpr int kMaxColTiles = 512;
 constexpr int kMaxTaps = 121;
 constexpr int kMaxCluster = 16;
@@ -458,12 +462,13 @@ __device__ __forceinline__ bool issue_segment(Bars* bars, uint64_t b0, uint64_t 
 }
 
 template <int N, bool PAIR, bool CONV, bool VEC, bool SWAP>
-__global__ void __launch_bounds__(kThreads, 1) shift_mma_kernel(const __grid_constant__ MmaSet S) {
+__global__ void __launch_bounds__(cta_threads(SWAP), 1) shift_mma_kernel(const __grid_constant__ MmaSet S) {
   using L = Layout<N, PAIR>;
   constexpr int NL = L::NL;            // columns whose weights this CTA decodes
   constexpr int kAccBufs = 128 / N;
   constexpr int kGroupSize = PAIR ? 2 : 1;
-  constexpr int kBSlotWarps = kBWarps / 2;  // B warps per slot
+  constexpr int kBWarps = b_warps(SWAP), kBSlotWarps = SWAP ? 4 : 2;  // B warps in all and per slot
+  constexpr int kThreads = cta_threads(SWAP), kMmaWarp = kFirstB + kBWarps;
   extern __shared__ __align__(1024) unsigned char smem[];
   Bars* bars = reinterpret_cast<Bars*>(smem);
   uint8_t* flags = smem + kFlagOff;
@@ -1166,29 +1171,24 @@ __global__ void __launch_bounds__(kThreads, 1) shift_mma_kernel(const __grid_con
         }
       }
     } else if (warp < kMmaWarp) {
-      const int bwarp = warp - kFirstB;
-      // ---- operand B: two groups of four warps take turns on the slots; a thread decodes 8 codes of one
-      // column (NL = 64), or the 4 even or odd ones of them (NL = 32) ----
-      constexpr int kGroups = 2;
-      constexpr bool kBoth = NL == 64;
-      static_assert(kGroups <= kSlots, "a group sees every use of its slots, so that phase parities suffice");
-      const int tb = (bwarp % kBSlotWarps) * 32 + lane;
-      const int g = bwarp / kBSlotWarps, h = g & 1;
-      const int col = tb % NL, kw = kBoth ? tb / NL : (tb / NL) >> 1;  // kw: which 8 of the slot's 16 indices
-      const int odd = kBoth ? 0 : (tb / NL) & 1;
+      // ---- operand B: three groups of two warps, group g fills ring slot g; a thread decodes 16 codes of one
+      // column (NL = 64) or 8 of them (NL = 32) ----
+      constexpr int kWords = NL / 32;  // code words of 8 indices
+      const int bwarp = warp - kFirstB, tb = (bwarp & 1) * 32 + lane;
+      slot = bwarp >> 1;
+      if (pass == 0) it = (uint32_t)slot;
+      const int col = tb % NL, kw = tb / NL;  // kw: which 8 of the slot's 16 indices (NL = 32)
       const uint32_t lut_a = tc::smem_u32(lut) + (lane & 7) * 16;
-      const uint32_t dst0 = tc::smem_u32(bslots) + col * 16 + (kw * 8 + odd) * NL * 16;
-      const uint32_t dig0 = tc::smem_u32(bdigits) + col * 16 + kw * 8 + odd * 4 + h * NL * 16;
-      if (pass == 0) {
-        it = (uint32_t)g;
-        slot = g % kSlots;
-        ring = (uint32_t)(g / kSlots) & 1u;
-      }
-      const uint32_t* nsrc = nullptr;  // the next load, as in operand A's warps
-      const uint2* bsrc = nullptr;
-      int rem = 0;
-      int64_t step = 0;
+      const uint32_t dst0 = tc::smem_u32(bslots) + slot * L::slot_bytes + col * 16 + kw * 8 * NL * 16;
+      const uint32_t dig0 = tc::smem_u32(bdigits) + col * 16 + kw * 8;
+      // The codes arrive kCodeAhead slots of the group ahead, in a ring of this
+      // thread's own words: 16 or 8 codes, sign and non-zero plane.
+      uint4* cells = reinterpret_cast<uint4*>(codes) + bwarp * 32 + lane;
+      uint32_t issued = 0, used = 0, modes = 0;  // modes, per slot in flight: bounded flag, half of the chunk
+      int rem = 0, half = 0;                     // the next load, as in operand A's warps
       uint32_t bounded = 0, in = 0;
+      int64_t cols = 0;
+      const unsigned char *nsrc = nullptr, *bsrc = nullptr;
       auto seek = [&](bool first, int n) {
         Walk<kGroupSize, SWAP> v(S, flags, digits, split ? pass : -1);
         bool more = true;
@@ -1207,31 +1207,34 @@ __global__ void __launch_bounds__(kThreads, 1) shift_mma_kernel(const __grid_con
         if (!more) return false;
         const GemmParams& P = v.P();
         const int64_t c = (int64_t)v.ct * N + cta * NL + col;
-        step = P.cols * (kGroups / 2);
-        in = c < P.cols;
-        bounded = v.fl & kBounded;
+        cols = P.cols;
+        in = c < cols;
+        bounded = (v.fl & kBounded) ? 1u : 0u;
         rem = 2 * (v.c_end - v.chunk) - n;
-        const int64_t rec = (int64_t)(v.chunk + (n >> 1)) * P.cols + (in ? c : 0);
-        nsrc = reinterpret_cast<const uint32_t*>(P.blob + P.off_nib + rec * 16) + 2 * h + kw;
-        bsrc = reinterpret_cast<const uint2*>(P.blob + P.off_bits + rec * 8);
+        half = n & 1;
+        const int64_t rec = (int64_t)(v.chunk + (n >> 1)) * cols + (in ? c : 0);
+        nsrc = P.blob + P.off_nib + rec * 16 + 4 * kw;
+        bsrc = P.blob + P.off_bits + rec * 8;
         return true;
       };
-      // The codes arrive kCodeAhead slots of the group ahead, in a ring of this
-      // thread's own words: 8 codes, sign and non-zero plane, bounded flag.
-      uint32_t* ring0 = reinterpret_cast<uint32_t*>(codes) + (bwarp * 32 + lane) * 4;
-      uint32_t issued = 0, used = 0;
       bool more = seek(true, (int)it);
       auto issue = [&]() {
         if (more) {
-          uint32_t* cell = ring0 + (issued % kCodeAhead) * kBWarps * 32 * 4;
-          cp_async8(cell, in ? (const void*)bsrc : (const void*)S.p[0].blob, in);
-          cp_async4(cell + 2, in ? (const void*)nsrc : (const void*)S.p[0].blob, in);
-          cell[3] = bounded;
+          unsigned char* cell = reinterpret_cast<unsigned char*>(cells + (issued % kCodeAhead) * 32 * kBWarps);
+          if constexpr (kWords == 2)
+            cp_async8(cell, in ? nsrc + 8 * half : S.p[0].blob, in);
+          else
+            cp_async4(cell, in ? nsrc + 8 * half : S.p[0].blob, in);
+          cp_async8(cell + 8, in ? bsrc : S.p[0].blob, in);
+          const uint32_t m = 1u << (issued % kCodeAhead), hm = m << 8;
+          modes = (modes & ~(m | hm)) | (bounded ? m : 0u) | (half ? hm : 0u);
           ++issued;
-          rem -= kGroups;
+          rem -= kSlots;
           if (rem > 0) {
-            nsrc += 4 * step;
-            bsrc += step;
+            half += kSlots;
+            nsrc += (half >> 1) * cols * 16;
+            bsrc += (half >> 1) * cols * 8;
+            half &= 1;
           } else {
             more = seek(false, -rem);
           }
@@ -1244,54 +1247,39 @@ __global__ void __launch_bounds__(kThreads, 1) shift_mma_kernel(const __grid_con
         issue();  // into the cell read in the previous turn
         if (used == issued) break;
         cp_async_wait<kCodeAhead - 1>();
-        const uint4 cell = *reinterpret_cast<const uint4*>(ring0 + (used % kCodeAhead) * kBWarps * 32 * 4);
+        const uint4 cell = cells[(used % kCodeAhead) * 32 * kBWarps];
+        const bool bnd = (modes >> (used % kCodeAhead)) & 1u;
+        const int h = (modes >> (8 + used % kCodeAhead)) & 1u;
         ++used;
-        const uint32_t nib = cell.z;
-        const uint2 bits = make_uint2(cell.x, cell.y);
-        const bool bnd = cell.w != 0;
-        const uint32_t b = (uint32_t)(16 * h + 8 * kw);
-        const uint32_t sb = bits.x >> (b + odd), zb = ~bits.y >> (b + odd);
-        // even (NL = 32: even or odd) codes
-        const uint32_t ne = ~(nib >> (4 * odd)) & 0x0F0F0F0Fu, se = spread(sb), ze = spread(zb);
-        uint32_t no = 0, so = 0, zo = 0;
-        uint32_t hi[2], lo[2], n3[2];
-        digit_weights(ne, se, ze, bnd, hi[0], lo[0], n3[0]);
-        if constexpr (kBoth) {
-          no = ~(nib >> 4) & 0x0F0F0F0Fu;
-          so = spread(sb >> 1);
-          zo = spread(zb >> 1);
-          digit_weights(no, so, zo, bnd, hi[1], lo[1], n3[1]);
-        }
         const uint32_t la = lut_a + (bnd ? 0 : kLutBytes);
-        const uint32_t dst = dst0 + slot * L::slot_bytes;
-        if (!wait(&bars->empty[slot], ring ^ 1u, abort)) break;
-        decode4<2 * NL * 16>(ne, se, ze, la, dst);
         // digit weights: [buffer][hi, lo, n3][16-index half][column][16 bytes]
-        const uint32_t dd = dig0 + ((it >> 1) & 1) * 3 * L::digit_bytes;
-        if constexpr (kBoth) {
+        const uint32_t dd = dig0 + ((it >> 1) & 1) * 3 * L::digit_bytes + h * NL * 16;
+        if (!wait(&bars->empty[slot], ring ^ 1u, abort)) break;
+#pragma unroll
+        for (int w8 = 0; w8 < kWords; ++w8) {
+          const uint32_t nib = w8 ? cell.y : cell.x, b = (uint32_t)(16 * h + 8 * (kw + w8));
+          const uint32_t sb = cell.z >> b, zb = ~cell.w >> b;
+          const uint32_t ne = ~nib & 0x0F0F0F0Fu, no = ~(nib >> 4) & 0x0F0F0F0Fu;
+          const uint32_t se = spread(sb), so = spread(sb >> 1), ze = spread(zb), zo = spread(zb >> 1);
+          const uint32_t dst = dst0 + w8 * 8 * NL * 16;
+          decode4<2 * NL * 16>(ne, se, ze, la, dst);
           decode4<2 * NL * 16>(no, so, zo, la, dst + NL * 16);
-          asm volatile("st.shared.v2.b32 [%0], {%1, %2};" ::"r"(dd), "r"(hi[0]), "r"(hi[1]) : "memory");
+          uint32_t hi[2], lo[2], n3[2];
+          digit_weights(ne, se, ze, bnd, hi[0], lo[0], n3[0]);
+          digit_weights(no, so, zo, bnd, hi[1], lo[1], n3[1]);
+          asm volatile("st.shared.v2.b32 [%0], {%1, %2};" ::"r"(dd + 8 * w8), "r"(hi[0]), "r"(hi[1]) : "memory");
           if (!bnd) {
-            asm volatile("st.shared.v2.b32 [%0], {%1, %2};" ::"r"(dd + L::digit_bytes), "r"(lo[0]), "r"(lo[1]) : "memory");
-            asm volatile("st.shared.v2.b32 [%0], {%1, %2};" ::"r"(dd + 2 * L::digit_bytes), "r"(n3[0]), "r"(n3[1]) : "memory");
-          }
-        } else {
-          asm volatile("st.shared.b32 [%0], %1;" ::"r"(dd), "r"(hi[0]) : "memory");
-          if (!bnd) {
-            asm volatile("st.shared.b32 [%0], %1;" ::"r"(dd + L::digit_bytes), "r"(lo[0]) : "memory");
-            asm volatile("st.shared.b32 [%0], %1;" ::"r"(dd + 2 * L::digit_bytes), "r"(n3[0]) : "memory");
+            asm volatile("st.shared.v2.b32 [%0], {%1, %2};" ::"r"(dd + 8 * w8 + L::digit_bytes), "r"(lo[0]), "r"(lo[1])
+                         : "memory");
+            asm volatile("st.shared.v2.b32 [%0], {%1, %2};" ::"r"(dd + 8 * w8 + 2 * L::digit_bytes), "r"(n3[0]), "r"(n3[1])
+                         : "memory");
           }
         }
         tc::fence_smem_async();
         __syncwarp();
         if (lane == 0) arrive(&bars->full[slot]);
-        it += kGroups;
-        slot += kGroups % kSlots;
-        ring ^= (uint32_t)(kGroups / kSlots) & 1u;
-        if (slot >= kSlots) {
-          slot -= kSlots;
-          ring ^= 1u;
-        }
+        it += kSlots;
+        ring ^= 1u;
       }
     } else if (cta == 0) {
       // ---- tensor operations (slot: chunks so far mod 3; it: digit buffer; ring: a bit per slot) ----
@@ -1480,7 +1468,7 @@ int max_clusters(int cs) {
   if (cache[cs] == 0) {
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3((unsigned)cs);
-    cfg.blockDim = dim3(kThreads);
+    cfg.blockDim = dim3(cta_threads(SWAP));
     cfg.dynamicSmemBytes = 200 * 1024;
     cudaLaunchAttribute attr;
     attr.id = cudaLaunchAttributeClusterDimension;
@@ -1525,7 +1513,7 @@ cudaError_t launch_n(MmaSet& S, int tiles, cudaStream_t st) {
   const size_t smem = Layout<N, PAIR>::total(S.table_entries, S.n, CONV);
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3((unsigned)((S.splits > 1 ? tiles * S.splits : std::min(tiles, units)) * group));
-  cfg.blockDim = dim3(kThreads);
+  cfg.blockDim = dim3(cta_threads(SWAP));
   cfg.dynamicSmemBytes = smem;
   cfg.stream = st;
   cudaLaunchAttribute attr;
