@@ -28,8 +28,11 @@ import synth_inputs as si  # noqa: E402
 METRIC = "Gshift-ops/s"
 L2_BYTES = 129 * 1024 * 1024
 INT_OPS_PER_CLK_PER_SM = 128  # 4 SMSPs x 32 lanes: 16-lane ALU pipe + 16-lane FMA pipe (IMAD)
+# The tensor-core kernels: a term is 17 fp8 multiply-adds (16 bit features of x and one digit), at 8192 a clock and
+# SM (tcgen05 kind::f8f6f4, 64.1 clocks measured for 128 x 128 x 32), so 2 int ops per 17 of them.
+TENSOR_INT_OPS_PER_CLK_PER_SM = 2 * 8192 / 17
 ALG_INT_OPS_PER_TERM = 2      # one shift + one add/subtract per term (Fig. 1a: MAC -> shift + add)
-# DRAM bytes (read + write) of one conv_direct_kernel<1,3,7,0> launch on this workload, from one ncu capture
+# DRAM bytes (read + write) of one shift_mma_kernel<64,1,1,0,0> launch on this workload, from one ncu capture
 # of the current kernel (dram__bytes_read.sum + dram__bytes_write.sum); y stays in L2 at kernel end.
 NCU_TRAFFIC_BYTES = 26.08e6
 HBM_NOMINAL_GBS = 7900.0  # GB300 HBM3e, nominal
@@ -129,6 +132,12 @@ def alu_peak(dev=None):
     peaks, kind = measured_peaks()
     sm_max = float(peaks.get("sm_max_mhz", 2070.0))
     return sms * INT_OPS_PER_CLK_PER_SM * sm_max * 1e6 / 1e12, sms, sm_max, kind
+
+
+def tensor_peak(dev=None):
+    """The same roofline for the tensor-core kernels: (T int-op equivalents/s, SMs, SM MHz, peak source)."""
+    tops, sms, sm_max, kind = alu_peak(dev)
+    return tops * TENSOR_INT_OPS_PER_CLK_PER_SM / INT_OPS_PER_CLK_PER_SM, sms, sm_max, kind
 
 
 def smi_gpu_id(index: int, visible: str | None) -> str:
@@ -355,7 +364,7 @@ def run_gpu_other(args, wl, rank, world, local_rank):
     clocks = sampler.stop()
     ms = e0.elapsed_time(e1)
     peaks, _ = measured_peaks()
-    alu_tops = alu_peak(dev)[0]
+    alu_tops = tensor_peak(dev)[0]
     value = terms * args.steps / (ms / 1e3) / 1e9
     if wl["kind"] == "fc16":
         tflops = 2 * terms / (ms / args.steps / 1e3) / 1e12
@@ -363,7 +372,7 @@ def run_gpu_other(args, wl, rank, world, local_rank):
         roof = {"bound": "tensor", "achieved": tflops, "peak": peak, "unit": "TFLOP/s", "frac": tflops / peak,
                 "traffic": None, "kernel": "linear_bf16_kernel", "peak_basis": "bf16_tflops (burst), measured"}
     else:
-        roof = {"bound": "alu", "achieved": 2 * terms / (ms / args.steps / 1e3) / 1e12, "peak": alu_tops,
+        roof = {"bound": "tensor", "achieved": 2 * terms / (ms / args.steps / 1e3) / 1e12, "peak": alu_tops,
                 "unit": "Tintop/s", "frac": 2 * terms / (ms / args.steps / 1e3) / 1e12 / alu_tops,
                 "traffic": None, "kernel": "whole step"}
     out = {"metric": METRIC, "value": value, "unit": METRIC, "n_gpus": 1, "steps": args.steps, "warmup": args.warmup,
@@ -484,7 +493,7 @@ def time_fc_layer(args, ds, dev, seed, M, K, N, backward=False):
     ms = e0.elapsed_time(e1) / reps
     terms = M * K * N
     return dict(shape=f"FC {K}->{N}", terms=terms, ms=ms, gsops=terms / ms / 1e6,
-                frac=2 * terms / (ms / 1e3) / (alu_peak(dev)[0] * 1e12))
+                frac=2 * terms / (ms / 1e3) / (tensor_peak(dev)[0] * 1e12))
 
 
 def run_specialized(args, wl, local_rank):
@@ -626,7 +635,7 @@ def run_layer_sweep(args, wl, local_rank):
         ms = e0.elapsed_time(e1) / reps
         terms = B * sp.K * OH * OW * sp.C * sp.R * sp.S
         r = dict(layer=i, shape=f"{sp.C}x{sp.H}x{sp.W}->{sp.K} {sp.R}x{sp.S}/{sp.stride}", terms=terms, ms=ms,
-                 gsops=terms / ms / 1e6, frac=2 * terms / (ms / 1e3) / (alu_peak(dev)[0] * 1e12))
+                 gsops=terms / ms / 1e6, frac=2 * terms / (ms / 1e3) / (tensor_peak(dev)[0] * 1e12))
         seen[key] = r
         rows.append(r)
         tot_terms += terms
@@ -675,7 +684,7 @@ def resnet18_forward_record(args, dev):
         torch.cuda.synchronize()
         ms = e0.elapsed_time(e1) / reps
         terms = PN.shift_terms(specs, batch)
-        alu_tops = alu_peak(dev)[0]
+        alu_tops = tensor_peak(dev)[0]
         rec[f"batch{batch}"] = {"ms_per_forward": ms, "gshift_ops_per_s": terms / ms / 1e6,
                                 "frac": 2 * terms / (ms / 1e3) / (alu_tops * 1e12), "terms": terms,
                                 # the program's ops and the max|x| pre-pass; a split layer adds a finalize
@@ -709,12 +718,12 @@ def sustained_record(step, n_rot, wl, dev, local_rank, seconds: float = 2.5):
     torch.cuda.synchronize()
     clocks = sampler.stop()
     ms = e0.elapsed_time(e1)
-    alu_tops, sms, sm_max, _ = alu_peak(dev)
+    alu_tops, sms, sm_max, _ = tensor_peak(dev)
     rate = wl["terms"] * n / (ms / 1e3)
     rec = {"steps": n, "seconds": ms / 1e3, "gshift_ops_per_s": rate / 1e9, "clocks": clocks,
            "frac": 2 * rate / (alu_tops * 1e12), "l2": f"rotating {n_rot} input/output sets, as the timed steps"}
     if clocks.get("sm_mhz"):
-        rec["frac_at_median_clock"] = 2 * rate / (sms * INT_OPS_PER_CLK_PER_SM * clocks["sm_mhz"] * 1e6)
+        rec["frac_at_median_clock"] = 2 * rate / (sms * TENSOR_INT_OPS_PER_CLK_PER_SM * clocks["sm_mhz"] * 1e6)
         rec["shift_ops_per_sm_clock"] = rate / (sms * clocks["sm_mhz"] * 1e6)
     return rec
 
@@ -850,7 +859,7 @@ def run_gpu(args, wl, rank, world, local_rank):
         peaks, peak_kind = measured_peaks()
         terms_total = wl["terms"] * args.steps * world
         value = terms_total / (ms_total / 1e3) / 1e9
-        alu_tops, sms, sm_max, _ = alu_peak(dev)  # T int-ops/s
+        alu_tops, sms, sm_max, _ = tensor_peak(dev)  # T int-ops/s
         achieved = ALG_INT_OPS_PER_TERM * wl["terms"] / (kern_ms / 1e3) / 1e12
         alg_bytes = 4 * (N * C * H * W + N * K * H * W) + ds.ds_packed_weight_bytes(K, C * R * S) + 4 * K
         out = {
@@ -862,10 +871,10 @@ def run_gpu(args, wl, rank, world, local_rank):
                        "activations": "uniform [0, 2^20) int32 Q16.16",
                        "l2": f"rotating {n_rot} input/output sets ({n_rot * per_step_bytes / 2**20:.0f} MiB > L2)",
                        "step": "absmax pre-pass + ConvShift (fused bias/saturate epilogue)"},
-            "roofline": {"bound": "alu", "achieved": achieved, "peak": alu_tops, "unit": "Tintop/s",
+            "roofline": {"bound": "tensor", "achieved": achieved, "peak": alu_tops, "unit": "Tintop/s",
                          "frac": achieved / alu_tops, "traffic": NCU_TRAFFIC_BYTES,
-                         "kernel": "conv_direct_kernel<1,3,7,0>", "kernel_ms": kern_ms,
-                         "peak_basis": f"{sms} SMs x {INT_OPS_PER_CLK_PER_SM} int32 ops/clk x {sm_max:.0f} MHz "
+                         "kernel": "shift_mma_kernel<64,1,1,0,0>", "kernel_ms": kern_ms,
+                         "peak_basis": f"{sms} SMs x 8192 fp8 multiply-adds/clk x {sm_max:.0f} MHz at 17 a term "
                                        f"(sm_max_mhz, {peak_kind})",
                          "alg_int_ops_per_launch": ALG_INT_OPS_PER_TERM * wl["terms"],
                          "hbm_gbs": alg_bytes / (kern_ms / 1e3) / 1e9,

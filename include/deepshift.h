@@ -83,8 +83,8 @@ size_t ds_abi_struct_size(int which);
 #define DS_AMAX_OUT 4u  /* write max|y| over this call's outputs into amax_io[1] */
 #define DS_RESIDUAL 8u  /* conv only: y = sat32(sat32(conv) + residual) before the ReLU */
 #define DS_FORCE_INT64 16u /* always use the 64-bit accumulator path (testing / worst case) */
-#define DS_CONV_IM2COL 32u /* conv only: use the implicit-GEMM (im2col gather) kernel instead of the
-                              direct halo-tile kernel (testing / comparison) */
+#define DS_CONV_IM2COL 32u /* conv only: use the implicit-GEMM (im2col gather) kernel on the CUDA cores
+                              instead of the tensor-core or halo-tile kernels (testing / comparison) */
 
 /* ---------------------------------------------------------------------------
  * Packed weights.
@@ -257,8 +257,9 @@ ds_status ds_expand_shift_weights_bf16(ds_weights* w, void* buf, size_t bytes, v
 ds_status ds_linear_shift_bf16(const uint16_t* x, const ds_weights* w, const float* bias, float* y, int64_t M,
                                int64_t K, int64_t N, uint32_t flags, void* stream);
 
-/* 1 if a bounded wait of the float kernel gave up in any ds_linear_shift_bf16 launch since the previous call of
- * this function (or since the library loaded), 0 if none did, -1 if the flag could not be read.  Reading clears
+/* 1 if a bounded wait of the float kernel, or of the integer tensor-core kernel (large ds_linear_shift and
+ * ds_conv2d_shift calls and their gradients), gave up in any launch since the previous call of this function (or
+ * since the library loaded), 0 if none did, -1 if the flag could not be read.  Reading clears
  * the flag.  The flag is device-wide and not per call: synchronise the streams of the calls it should cover
  * first (the read itself is a synchronous copy).  A launch whose wait gave up stops early, so its y is
  * incomplete.  A library utility: no counterpart in the paper. */

@@ -41,14 +41,14 @@
 // CTA: 128 rows (tensor-memory lanes) x N columns; a pair of CTAs shares a tile
 // of 256 rows, each decoding half of its weights (cta_group::2), since a tile's
 // weight bytes are written to and read from shared memory once per 128 or 256
-// rows.  25 warps, with x as operand A:
+// rows.  23 warps (swapped roles, below: 25), with x as operand A:
 //   warps 0-11   operand A, three groups of four: a thread gathers 16 values of
 //                its row, expands them and writes them to tensor memory
 //   warps 12-15  epilogue: accumulators to integer sums in shared memory, then
 //                bias, saturation, residual, ReLU, max|y| and the output
-//   warps 16-23  operand B, two groups of four: decode the packed codes of a
+//   warps 16-21  operand B, three groups of two: decode the packed codes of a
 //                column through a table of weight bytes into shared memory
-//   warp 24      issues the tensor operations
+//   warp 22      issues the tensor operations
 // FC layers of up to 128 rows swap the operands' roles: the lanes are 128 weight
 // columns, decoded into tensor memory, and N = 64 rows of x are expanded into
 // shared memory, so that no lane is idle and a code is decoded once per 64 rows
@@ -60,9 +60,14 @@
 // expiry the CTA stops and sets a flag.
 //
 // Measured (GB300, per call with the max|x| pre-pass, against the CUDA-core
-// kernels): FC 8192 x 4096 x 4096 9.94 -> 1.56 ms, ConvShift 64x56x56 3x3 at batch
-// 32 0.296 -> 0.143 ms, 256x14x14 -> 512 3x3/2 0.216 -> 0.066 ms, 1024x14x14 -> 256
-// 1x1 at batch 64 0.301 -> 0.104 ms.
+// kernels): FC 8192 x 4096 x 4096 9.94 -> 1.46 ms (about 760 clocks a slot of 16
+// indices; the operations alone take 608), ConvShift 64x56x56 3x3 at batch 32 0.296
+// -> 0.124 ms, 256x14x14 -> 512 3x3/2 0.216 -> 0.058 ms, 1024x14x14 -> 256 1x1 at batch
+// 64 0.301 -> 0.096 ms, VGG16 FC1 at batch 64 0.565 -> 0.206 ms.  What bounds it: at
+// N = 128 the ALU pipe (expanding x: 5-6 of its instructions a value, which run
+// at 64 lanes a clock and SM) and the operations' issue; at N = 64 the issuing
+// warp (about 590 clocks a slot with nothing else done, against 272 of
+// operations) and operand A.  wait -> issue -> commit is a chain of single instructions.
 #include <cooperative_groups.h>
 
 #include <algorithm>
@@ -1526,7 +1531,7 @@ cudaError_t launch_n(MmaSet& S, int tiles, cudaStream_t st) {
   return cudaLaunchKernelEx(&cfg, shift_mma_kernel<N, PAIR, CONV, VEC, SWAP>, S);
 }
 
-template <int N, bool PAIR, bool SWAP = false>
+template <int N, bool PAIR, bool SWAP = !PAIR>
 cudaError_t launch_set(const GemmParams* ps, int n, bool conv, cudaStream_t st) {
   MmaSet S{};
   S.n = n;
@@ -1596,8 +1601,7 @@ cudaError_t launch_shift_mma(const GemmParams* ps, int n, bool conv, cudaStream_
     cols = std::max(cols, ps[i].cols);
     rows = std::max(rows, ps[i].rows);
   }
-  if (!conv && rows <= kRows) return launch_set<64, false, true>(ps, n, conv, st);
-  if (rows <= kRows) return launch_set<64, false>(ps, n, conv, st);
+  if (!conv && rows <= kRows) return launch_set<64, false>(ps, n, false, st);  // few rows: swapped roles
   return cols <= 64 ? launch_set<64, true>(ps, n, conv, st) : launch_set<128, true>(ps, n, conv, st);
 }
 
