@@ -48,7 +48,7 @@
 //                bias, saturation, residual, ReLU, max|y| and the output
 //   warps 16-21  operand B, three groups of two: decode the packed codes of a
 //                column through a table of weight bytes into shared memory
-//   warp 22      issues the tensor operations
+//   warp 22      issues the tensor operations (swapped roles: warp 16, B after it)
 // FC layers of up to 128 rows swap the operands' roles: the lanes are 128 weight
 // columns, decoded into tensor memory, and N = 64 rows of x are expanded into
 // shared memory, so that no lane is idle and a code is decoded once per 64 rows
@@ -62,8 +62,8 @@
 // Measured (GB300, per call with the max|x| pre-pass, against the CUDA-core
 // kernels): FC 8192 x 4096 x 4096 9.94 -> 1.46 ms (about 760 clocks a slot of 16
 // indices; the operations alone take 608), ConvShift 64x56x56 3x3 at batch 32 0.296
-// -> 0.124 ms, 256x14x14 -> 512 3x3/2 0.216 -> 0.058 ms, 1024x14x14 -> 256 1x1 at batch
-// 64 0.301 -> 0.096 ms, VGG16 FC1 at batch 64 0.565 -> 0.206 ms.  What bounds it: at
+// -> 0.116 ms, 256x14x14 -> 512 3x3/2 0.216 -> 0.058 ms, 1024x14x14 -> 256 1x1 at batch
+// 64 0.301 -> 0.096 ms, VGG16 FC1 at batch 64 0.565 -> 0.193 ms.  What bounds it: at
 // N = 128 the ALU pipe (expanding x: 5-6 of its instructions a value, which run
 // at 64 lanes a clock and SM) and the operations' issue; at N = 64 the issuing
 // warp (about 590 clocks a slot with nothing else done, against 272 of
@@ -98,7 +98,13 @@ constexpr int kFirstEpi = kAWarps, kFirstB = kFirstEpi + kEpiWarps;
 // warps leave a thread 80 registers, 25 leave 72: with 72 the convolution's operand
 // A spills in its loop (a version with 270 spilled bytes ran 15-30% slower).
 __host__ __device__ constexpr int b_warps(bool swap) { return swap ? 8 : 6; }
-__host__ __device__ constexpr int cta_threads(bool swap) { return 32 * (kFirstB + b_warps(swap) + 1); }
+__device__ __forceinline__ int swapped_b_warp(int warp) {
+  return warp > kFirstB && (warp & 3) != 0 ? 3 * ((warp - kFirstB) >> 2) + (warp & 3) - 1 : 1 << 16;
+}
+// Swapped roles: the issuing warp is warp 16 and B's are 17-19, 21-23, 25 and 26 (20
+// and 24 idle), so that no B warp is on its scheduler: VGG16 FC1 at batch 64 0.206
+// -> 0.193 ms.  (Unswapped, the two more warps would cost the 80 registers.)
+__host__ __device__ constexpr int cta_threads(bool swap) { return 32 * (swap ? 27 : kFirstB + b_warps(false) + 1); }
 constexpr int kCodeAhead = 4;   // slots of a B group whose codes are in flight
 constexpr int kCodeBytes = kCodeAhead * b_warps(false) * 32 * 16;
 constexpr int kMaxColTiles = 512;
@@ -473,7 +479,7 @@ __global__ void __launch_bounds__(cta_threads(SWAP), 1) shift_mma_kernel(const _
   constexpr int kAccBufs = 128 / N;
   constexpr int kGroupSize = PAIR ? 2 : 1;
   constexpr int kBWarps = b_warps(SWAP), kBSlotWarps = SWAP ? 4 : 2;  // B warps in all and per slot
-  constexpr int kThreads = cta_threads(SWAP), kMmaWarp = kFirstB + kBWarps;
+  constexpr int kThreads = cta_threads(SWAP), kMmaWarp = SWAP ? kFirstB : kFirstB + kBWarps;
   extern __shared__ __align__(1024) unsigned char smem[];
   Bars* bars = reinterpret_cast<Bars*>(smem);
   uint8_t* flags = smem + kFlagOff;
@@ -1057,9 +1063,9 @@ __global__ void __launch_bounds__(cta_threads(SWAP), 1) shift_mma_kernel(const _
         ++seg_no;
         more = next_segment_or_tile(w);
       }
-    } else if (SWAP && warp < kMmaWarp) {
+    } else if (SWAP && swapped_b_warp(warp) < kBWarps) {
       // ---- operand B, swapped roles: two groups of four warps; a thread expands 8 values of one row of x ----
-      const int tb = (warp - kFirstB) % kBSlotWarps * 32 + lane, g = (warp - kFirstB) / kBSlotWarps;
+      const int bwarp = swapped_b_warp(warp), tb = bwarp % kBSlotWarps * 32 + lane, g = bwarp / kBSlotWarps;
       const int n = tb % N, kw = tb / N;  // row of the tile, which 8 of the slot's 16 indices
       static_assert(!SWAP || N == 64, "128 threads: 64 rows x 16 indices");
       const uint32_t dst0 = tc::smem_u32(bslots) + n * 16 + kw * 8 * N * 16;
@@ -1069,7 +1075,7 @@ __global__ void __launch_bounds__(cta_threads(SWAP), 1) shift_mma_kernel(const _
         slot = g;
       }
       // kCodeAhead slots of 8 values, in flight to this thread's own words
-      int4* cells = reinterpret_cast<int4*>(xrows + kCodeAhead * kAWarps * 32 * 16) + ((warp - kFirstB) * 32 + lane);
+      int4* cells = reinterpret_cast<int4*>(xrows + kCodeAhead * kAWarps * 32 * 16) + (bwarp * 32 + lane);
       uint32_t issued = 0, used = 0, modes = 0;  // modes: a byte per slot in flight: bounded flag, digit
       int rem = 0, left = 0;
       uint32_t mode = 0;
@@ -1175,7 +1181,7 @@ __global__ void __launch_bounds__(cta_threads(SWAP), 1) shift_mma_kernel(const _
           ring ^= 1u;
         }
       }
-    } else if (warp < kMmaWarp) {
+    } else if (!SWAP && warp < kMmaWarp) {
       // ---- operand B: three groups of two warps, group g fills ring slot g; a thread decodes 16 codes of one
       // column (NL = 64) or 8 of them (NL = 32) ----
       constexpr int kWords = NL / 32;  // code words of 8 indices
@@ -1286,7 +1292,7 @@ __global__ void __launch_bounds__(cta_threads(SWAP), 1) shift_mma_kernel(const _
         it += kSlots;
         ring ^= 1u;
       }
-    } else if (cta == 0) {
+    } else if (warp == kMmaWarp && cta == 0) {
       // ---- tensor operations (slot: chunks so far mod 3; it: digit buffer; ring: a bit per slot) ----
       Walk<kGroupSize, SWAP> w(S, flags, digits, split ? pass : -1);
       w.start_tile();
