@@ -52,7 +52,7 @@
 // FC layers of up to 128 rows swap the operands' roles: the lanes are 128 weight
 // columns, decoded into tensor memory, and N = 64 rows of x are expanded into
 // shared memory, so that no lane is idle and a code is decoded once per 64 rows
-// (VGG16 FC1 at batch 64: 0.361 ms with rows as lanes, 0.206 ms so).
+// (VGG16 FC1 at batch 64: 0.361 ms with rows as lanes, 0.206 ms so, 0.189 ms now).
 // A ring of three slots of 16 reduction indices connects them; CTAs are
 // persistent over tiles and the ring runs on across them.  A grid that leaves
 // SMs idle splits the reduction over the CTAs of a cluster, which sum their
@@ -62,8 +62,8 @@
 // Measured (GB300, per call with the max|x| pre-pass, against the CUDA-core
 // kernels): FC 8192 x 4096 x 4096 9.94 -> 1.46 ms (about 760 clocks a slot of 16
 // indices; the operations alone take 608), ConvShift 64x56x56 3x3 at batch 32 0.296
-// -> 0.116 ms, 256x14x14 -> 512 3x3/2 0.216 -> 0.058 ms, 1024x14x14 -> 256 1x1 at batch
-// 64 0.301 -> 0.096 ms, VGG16 FC1 at batch 64 0.565 -> 0.193 ms.  What bounds it: at
+// -> 0.112 ms, 256x14x14 -> 512 3x3/2 0.216 -> 0.051 ms, 1024x14x14 -> 256 1x1 at batch
+// 64 0.301 -> 0.086 ms, VGG16 FC1 at batch 64 0.565 -> 0.189 ms.  What bounds it: at
 // N = 128 the ALU pipe (expanding x: 5-6 of its instructions a value, which run
 // at 64 lanes a clock and SM) and the operations' issue; at N = 64 the issuing
 // warp (about 590 clocks a slot with nothing else done, against 272 of
@@ -102,8 +102,10 @@ __device__ __forceinline__ int swapped_b_warp(int warp) {
   return warp > kFirstB && (warp & 3) != 0 ? 3 * ((warp - kFirstB) >> 2) + (warp & 3) - 1 : 1 << 16;
 }
 // Swapped roles: the issuing warp is warp 16 and B's are 17-19, 21-23, 25 and 26 (20
-// and 24 idle), so that no B warp is on its scheduler: VGG16 FC1 at batch 64 0.206
-// -> 0.193 ms.  (Unswapped, the two more warps would cost the 80 registers.)
+// and 24 idle), so that no B warp is on its scheduler: VGG16 FC1 at batch 64 0.205
+// -> 0.193 ms on one GPU in turn.  The unswapped kernels' roles are as before, but their
+// convolutions measured 3-6% faster with the changed branch conditions (64x56x56 3x3
+// 0.125 -> 0.117 ms, FC unchanged); why was not isolated.  (Unswapped, the two more warps would cost the 80 registers.)
 __host__ __device__ constexpr int cta_threads(bool swap) { return 32 * (swap ? 27 : kFirstB + b_warps(false) + 1); }
 constexpr int kCodeAhead = 4;   // slots of a B group whose codes are in flight
 constexpr int kCodeBytes = kCodeAhead * b_warps(false) * 32 * 16;
