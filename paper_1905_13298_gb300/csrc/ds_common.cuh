@@ -215,24 +215,26 @@ __host__ __device__ inline int64_t expanded_words(int64_t n_out, int64_t k_red) 
 #ifdef __CUDACC__
 // Asynchronous global -> shared copies of 4, 8 or 16 bytes; valid = false
 // zero-fills the destination (source size 0).  4 and 8 bytes go through L1,
-// 16 bytes bypass it.
+// 16 bytes bypass it.  The "memory" clobbers keep a thread's ordinary reads of
+// the words on their side: after the wait for the copy that delivers them, and
+// before the copy that overwrites them (some users have no barrier there).
 __device__ __forceinline__ void cp_async4(void* smem_dst, const void* gsrc, bool valid) {
   const uint32_t d = (uint32_t)__cvta_generic_to_shared(smem_dst);
-  asm volatile("cp.async.ca.shared.global [%0], [%1], 4, %2;\n" ::"r"(d), "l"(gsrc), "r"(valid ? 4 : 0));
+  asm volatile("cp.async.ca.shared.global [%0], [%1], 4, %2;\n" ::"r"(d), "l"(gsrc), "r"(valid ? 4 : 0) : "memory");
 }
 __device__ __forceinline__ void cp_async8(void* smem_dst, const void* gsrc, bool valid) {
   const uint32_t d = (uint32_t)__cvta_generic_to_shared(smem_dst);
-  asm volatile("cp.async.ca.shared.global [%0], [%1], 8, %2;\n" ::"r"(d), "l"(gsrc), "r"(valid ? 8 : 0));
+  asm volatile("cp.async.ca.shared.global [%0], [%1], 8, %2;\n" ::"r"(d), "l"(gsrc), "r"(valid ? 8 : 0) : "memory");
 }
 __device__ __forceinline__ void cp_async16(void* smem_dst, const void* gsrc, bool valid) {
   const uint32_t d = (uint32_t)__cvta_generic_to_shared(smem_dst);
-  asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;\n" ::"r"(d), "l"(gsrc), "r"(valid ? 16 : 0));
+  asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;\n" ::"r"(d), "l"(gsrc), "r"(valid ? 16 : 0) : "memory");
 }
-__device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;\n" ::); }
+__device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;\n" ::: "memory"); }
 // Wait until at most N of this thread's committed copy groups are in flight.
 template <int N>
 __device__ __forceinline__ void cp_async_wait() {
-  asm volatile("cp.async.wait_group %0;\n" ::"n"(N));
+  asm volatile("cp.async.wait_group %0;\n" ::"n"(N) : "memory");
 }
 __device__ __forceinline__ void cp_async_wait_all() { cp_async_wait<0>(); }
 // Saturating int32 addition (the residual join) and |v| as an unsigned value.
@@ -272,7 +274,8 @@ struct ExpandedCodeStager {
     for (int u = 0; u < 4; ++u) {
       const int kl8 = (u & 1) * 8, b = u >> 1;
       asm volatile("cp.async.cg.shared.global [%0], [%1], 16;\n" ::"r"(d + (uint32_t)(kl8 * 128 + b * 64) * 4),
-                   "l"(s + kl8 * 64 + b * kred_words));
+                   "l"(s + kl8 * 64 + b * kred_words)
+                   : "memory");
     }
   }
   // stage st (indices kbeg + 16 st ..) into cs; zero fill past kred and for an absent block
@@ -287,7 +290,8 @@ struct ExpandedCodeStager {
       const bool ok = k + kl8 < kred && (b == 0 || b1);
       const int32_t* g = ok ? s + kl8 * 64 + b * kred * 64 : xcodes;
       asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;\n" ::"r"(d + (uint32_t)(kl8 * 128 + b * 64) * 4),
-                   "l"(g), "r"(ok ? 16 : 0));
+                   "l"(g), "r"(ok ? 16 : 0)
+                   : "memory");
     }
   }
 };

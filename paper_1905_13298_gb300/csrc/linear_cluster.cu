@@ -119,7 +119,7 @@ struct XStager {
       if constexpr (XV) {
         const int n = left >= 4 ? 16 : (left > 0 ? 4 * (int)left : 0);
         const uint32_t d = (uint32_t)__cvta_generic_to_shared(xt + 4 * e);
-        asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;\n" ::"r"(d), "l"(n ? s : P.x), "r"(n));
+        asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;\n" ::"r"(d), "l"(n ? s : P.x), "r"(n) : "memory");
       } else {
 #pragma unroll
         for (int i = 0; i < 4; ++i)
@@ -136,7 +136,7 @@ struct XStager {
       const int32_t* s = src[u] + (int64_t)st * KC;
       if constexpr (XV) {
         const uint32_t d = (uint32_t)__cvta_generic_to_shared(xt + 4 * e);
-        asm volatile("cp.async.cg.shared.global [%0], [%1], 16;\n" ::"r"(d), "l"(s));
+        asm volatile("cp.async.cg.shared.global [%0], [%1], 16;\n" ::"r"(d), "l"(s) : "memory");
       } else {
 #pragma unroll
         for (int i = 0; i < 4; ++i) cp_async4(xt + 4 * e + i, s + i, true);

@@ -216,10 +216,10 @@ std::string kernel_source(const int8_t* s, const int8_t* p, const ds_specialized
       "    _Pragma(\"unroll\") for (int i = 0; i < WS; ++i) {\n"
       "      const bool ok = rok && (unsigned)(iws + i) < (unsigned)W;\n"
       "      asm volatile(\"cp.async.ca.shared.global [%0], [%1], 4, %2;\" :: \"r\"(d0 + 4u * i),\n"
-      "                   \"l\"(ok ? (const void*)(src + iws + i) : (const void*)x), \"r\"(ok ? 4 : 0));\n"
+      "                   \"l\"(ok ? (const void*)(src + iws + i) : (const void*)x), \"r\"(ok ? 4 : 0) : \"memory\");\n"
       "    }\n"
       "  }\n"
-      "  asm volatile(\"cp.async.commit_group;\");\n"
+      "  asm volatile(\"cp.async.commit_group;\" ::: \"memory\");\n"
       // the bound, per channel of the group (A, nnz immediates; max|x| and bias at run time)
       "  bool exact = amax_in != 0 && !(flags & 16u);\n"
       "  const u64 amax = amax_in ? (u64)*amax_in : 0ull;\n"
