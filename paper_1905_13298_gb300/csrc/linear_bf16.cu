@@ -31,6 +31,7 @@
 #include <cudaTypedefs.h>
 
 #include "ds_common.cuh"
+#include "tensor_core.cuh"
 
 namespace ds {
 
@@ -289,7 +290,7 @@ __global__ void __launch_bounds__(kThreads, 1)
               "=r"(r[29]), "=r"(r[30]), "=r"(r[31])
             : "r"(taddr)
             : "memory");
-        asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+        tc::wait_ld(r);
         if (c0 + 32 == BN) {
           // the whole accumulator is in registers: hand it back to the MMA warp
           asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");

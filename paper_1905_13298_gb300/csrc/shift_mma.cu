@@ -938,7 +938,7 @@ __global__ void __launch_bounds__(cta_threads(SWAP), 1) shift_mma_kernel(const _
           uint32_t rl[16], rh[16];
           tc::ld16(acc + c0, rl);
           tc::ld16(acc + N + c0, rh);
-          tc::wait_ld();
+          tc::wait_ld(rl, rh);
           if (i32) {
             uint32_t* a = acc32 + c0 * kAccStride;
 #pragma unroll

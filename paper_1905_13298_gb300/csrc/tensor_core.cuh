@@ -32,7 +32,18 @@ __device__ __forceinline__ void fence_before() { asm volatile("tcgen05.fence::be
 __device__ __forceinline__ void fence_after() { asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory"); }
 __device__ __forceinline__ void fence_smem_async() { asm volatile("fence.proxy.async.shared::cta;" ::: "memory"); }
 __device__ __forceinline__ void wait_st() { asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory"); }
-__device__ __forceinline__ void wait_ld() { asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory"); }
+// Waits for this thread's tensor-memory loads into r (any number of arrays).  The
+// loads write their registers up to here, so the registers take their values
+// here: without the empty statements arithmetic on them could move before the wait.
+template <int... N>
+__device__ __forceinline__ void wait_ld(uint32_t (&... r)[N]) {
+  asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+  auto take = [](auto& a) {
+#pragma unroll
+    for (auto& v : a) asm volatile("" : "+r"(v));
+  };
+  (take(r), ...);
+}
 
 // One lane of a converged warp (the same lane every time).
 __device__ __forceinline__ bool elect_one() {

@@ -37,3 +37,20 @@ def test_ordering_asm_has_a_memory_clobber(path):
         text = f.read().replace('\\"', '"') if path.endswith("specialize.cu") else f.read()
     missing = [line for line, s in _statements(text) if ORDERING.search(s) and '"memory"' not in s]
     assert missing == []
+
+
+def test_tensor_memory_loads_are_used_after_their_wait():
+    """A tensor-memory load writes its registers up to the wait: the one place that waits names them as rewritten."""
+    waits = {}
+    for path in glob.glob(os.path.join(CSRC, "*.cu*")):
+        with open(path) as f:
+            text = f.read()
+        n = text.count("tcgen05.wait::ld")
+        if n:
+            waits[os.path.basename(path)] = n
+        if os.path.basename(path) != "tensor_core.cuh":
+            assert not re.search(r"wait_ld\(\s*\)", text), path
+    assert waits == {"tensor_core.cuh": 1}
+    with open(os.path.join(CSRC, "tensor_core.cuh")) as f:
+        body = f.read().split("void wait_ld(", 1)[1].split("\n}\n", 1)[0]
+    assert '"+r"' in body
