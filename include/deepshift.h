@@ -262,11 +262,13 @@ ds_status ds_linear_shift_bf16(const uint16_t* x, const ds_weights* w, const flo
  * since the library loaded), 0 if none did, -1 if the flag could not be read.  Reading clears
  * the flag.  The flag is device-wide and not per call: synchronise the streams of the calls it should cover
  * first (the read itself is a synchronous copy).  A launch whose wait gave up stops early, so its y is
- * incomplete.  A library utility: no counterpart in the paper. */
+ * incomplete: outputs that it did not make are left as they were, and a max|y| that it reports (DS_AMAX_OUT) is 2^31.
+ * The call has returned DS_OK by then: a caller that must know reads this flag.  A library utility: no counterpart in
+ * the paper. */
 int ds_bf16_fault_flag(void);
 
-/* Diagnostic: the limit, in SM clock cycles, of each bounded wait of the float kernel's later launches; cycles <= 0
- * restores the default (4e9 cycles, about 2 s).  A launch whose wait runs out stops issuing work, lets the copies and
+/* Diagnostic: the limit, in SM clock cycles, of each bounded wait of later launches of the float kernel and of the
+ * integer tensor-core kernel; cycles <= 0 restores the default (4e9 cycles, about 2 s).  A launch whose wait runs out stops issuing work, lets the copies and
  * tensor-core operations it already issued finish, frees its tensor memory and sets the fault flag above, so a test
  * can make the waits run out on purpose and the context stays usable.  Process-wide (not per stream or thread).
  * A library utility: no counterpart in the paper. */

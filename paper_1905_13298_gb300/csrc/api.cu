@@ -433,7 +433,10 @@ int ds_bf16_fault_flag(void) {
   return a < 0 || b < 0 ? -1 : (a | b);
 }
 
-void ds_bf16_set_wait_limit(long long cycles) { set_bf16_wait_cycles(cycles); }
+void ds_bf16_set_wait_limit(long long cycles) {
+  set_bf16_wait_cycles(cycles);
+  set_mma_wait_cycles(cycles);
+}
 
 ds_status ds_linear_shift_backward_x(const int32_t* dy, const ds_weights* w_bwd, int32_t* dx, int64_t M, int64_t K,
                                      int64_t N, uint32_t flags, uint32_t* amax_io, void* stream) {

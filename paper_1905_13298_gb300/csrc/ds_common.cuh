@@ -137,6 +137,7 @@ cudaError_t launch_conv_narrow(const GemmParams& p, cudaStream_t st);
 bool shift_mma_preferred(const GemmParams* ps, int n, bool conv);
 cudaError_t launch_shift_mma(const GemmParams* ps, int n, bool conv, cudaStream_t st);
 int read_mma_fault_flag();
+void set_mma_wait_cycles(long long cycles);
 // Launchers (defined in shift_gemm.cu).
 cudaError_t launch_linear_shift(const GemmParams& p, cudaStream_t st);
 // Defined in linear_cluster.cu (small batches: the reduction split over a thread-block cluster).

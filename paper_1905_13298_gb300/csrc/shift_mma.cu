@@ -56,8 +56,10 @@
 // A ring of three slots of 16 reduction indices connects them; CTAs are
 // persistent over tiles and the ring runs on across them.  A grid that leaves
 // SMs idle splits the reduction over the CTAs of a cluster, which sum their
-// partial tiles through distributed shared memory.  Every wait is bounded; on
-// expiry the CTA stops and sets a flag.
+// partial tiles through distributed shared memory.  Every barrier wait of a role
+// is bounded; on expiry the CTA stops and sets a flag, and no output is made from
+// its sums.  The cluster barriers need no bound of their own: every CTA reaches
+// them, since its roles' waits are bounded.
 //
 // Measured (GB300, per call with the max|x| pre-pass, against the CUDA-core
 // kernels): FC 8192 x 4096 x 4096 9.94 -> 1.46 ms (about 760 clocks a slot of 16
@@ -71,6 +73,7 @@
 #include <cooperative_groups.h>
 
 #include <algorithm>
+#include <atomic>
 #include <mutex>
 #include <type_traits>
 
@@ -113,6 +116,10 @@ constexpr int kMaxColTiles = 512;
 constexpr int kMaxTaps = 121;
 constexpr int kMaxCluster = 16;
 constexpr long long kWaitCycles = 4000000000LL;  // about 2 s
+
+// the wait limit of the next launches (a diagnostic can shorten it to make the waits run out)
+std::atomic<long long> g_wait_cycles{kWaitCycles};
+
 constexpr int kAccStride = kRows + 1;  // words between a column's sums and the next one's: no bank conflicts either way
 constexpr int kXStride = 20;    // words per staged row of 16 values: 16-byte reads of 8 rows hit all banks
 
@@ -134,12 +141,14 @@ struct MmaSet {
   GemmParams p[kMaxGemmPhases];
   PhaseInfo info[kMaxGemmPhases];
   int n, splits, table_entries;  // table_entries: per phase
+  long long wait_cycles;         // limit of a barrier wait before the CTA gives up
 };
 
 struct __align__(8) Bars {
   uint64_t full[kSlots], empty[kSlots], acc_full[2], acc_empty[2], done;
+  long long wait_cycles;
   uint32_t tmem, amax;
-  int abort;
+  int abort;  // a wait of this CTA has given up
 };
 
 constexpr int kLutBytes = 64 * 128;
@@ -161,22 +170,22 @@ struct Layout {
   }
 };
 
-__device__ __noinline__ bool slow_wait(uint64_t* bar, uint32_t parity, volatile int* abort) {
+// A whole warp waits, and goes on or gives up as one: its lanes' looks at the
+// barrier may differ, and what follows is warp-wide tensor-memory work.
+__device__ __noinline__ bool slow_wait(uint64_t* bar, uint32_t parity, volatile Bars* bars) {
   const long long t0 = clock64();
   while (!tc::mbar_try_wait(bar, parity)) {
-    if (*abort) return false;
-    if (clock64() - t0 > kWaitCycles) {
-      *abort = 1;
+    if (bars->abort) return false;
+    if (clock64() - t0 > bars->wait_cycles) {
+      bars->abort = 1;
       atomicExch(&g_mma_fault, 1);
       return false;
     }
   }
   return true;
 }
-__device__ __forceinline__ bool wait(uint64_t* bar, uint32_t parity, volatile int* abort) {
-  const bool ok = tc::mbar_try_wait(bar, parity) || slow_wait(bar, parity, abort);
-  __syncwarp();
-  return ok;
+__device__ __forceinline__ bool wait(uint64_t* bar, uint32_t parity, volatile Bars* bars) {
+  return __all_sync(0xffffffffu, tc::mbar_try_wait(bar, parity) || slow_wait(bar, parity, bars));
 }
 
 // The walk over a CTA's tiles, and in each tile over its segments (column half,
@@ -440,15 +449,14 @@ __device__ __forceinline__ void issue_slot(uint64_t b0, uint64_t d0, bool dbuf, 
 template <int N, bool PAIR, bool SWAP, int BUF>
 __device__ __forceinline__ bool issue_segment(Bars* bars, uint64_t b0, uint64_t d0, int n, int& pos, uint32_t& ring,
                                               bool& dbuf, bool bounded, uint32_t pair_mask) {
-  volatile int* abort = &bars->abort;
   uint32_t first = 0;
   auto chunk = [&](auto p) {
     constexpr int S0 = 2 * decltype(p)::value % 3, S1 = (S0 + 1) % 3;
-    if (!wait(&bars->full[S0], (ring >> S0) & 1u, abort)) return false;
+    if (!wait(&bars->full[S0], (ring >> S0) & 1u, bars)) return false;
     tc::fence_after();
     if (tc::elect_one()) issue_slot<N, PAIR, SWAP, S0, BUF, false>(b0, d0, dbuf, first, bounded, bars->empty, pair_mask);
     __syncwarp();
-    if (!wait(&bars->full[S1], (ring >> S1) & 1u, abort)) return false;
+    if (!wait(&bars->full[S1], (ring >> S1) & 1u, bars)) return false;
     tc::fence_after();
     if (tc::elect_one()) issue_slot<N, PAIR, SWAP, S1, BUF, true>(b0, d0, dbuf, first, bounded, bars->empty, pair_mask);
     __syncwarp();
@@ -492,7 +500,6 @@ __global__ void __launch_bounds__(cta_threads(SWAP), 1) shift_mma_kernel(const _
   unsigned char* accs = bdigits + 6 * L::digit_bytes;
   unsigned char* codes = accs + L::acc_bytes;
   unsigned char* xrows = codes + kCodeBytes;
-  volatile int* abort = &bars->abort;
   const int tid = threadIdx.x, lane = tid & 31;
   const int warp = __shfl_sync(0xffffffffu, tid >> 5, 0);
   const int cta = PAIR ? (int)(blockIdx.x & 1) : 0;  // place in the pair: its rows of the tile
@@ -512,6 +519,7 @@ __global__ void __launch_bounds__(cta_threads(SWAP), 1) shift_mma_kernel(const _
     }
     tc::mbar_init(&bars->done, 1);
     bars->abort = 0;
+    bars->wait_cycles = S.wait_cycles;
     bars->amax = 0;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
@@ -691,7 +699,7 @@ __global__ void __launch_bounds__(cta_threads(SWAP), 1) shift_mma_kernel(const _
         const uint32_t la = lut_a + (bnd ? 0 : kLutBytes);
         const uint32_t sp = cell.z >> (16 * h), zp = ~cell.w >> (16 * h);
         const uint32_t ad = d0 + 12 * (it & 2) + 4 * h;
-        if (!wait(&bars->empty[slot], ring ^ 1u, abort)) break;
+        if (!wait(&bars->empty[slot], ring ^ 1u, bars)) break;
         tc::fence_after();
 #pragma unroll
         for (int w8 = 0; w8 < 2; ++w8) {
@@ -862,7 +870,7 @@ __global__ void __launch_bounds__(cta_threads(SWAP), 1) shift_mma_kernel(const _
           }
           __syncwarp();
         }
-        if (!wait(&bars->empty[slot], ring ^ 1u, abort)) break;
+        if (!wait(&bars->empty[slot], ring ^ 1u, bars)) break;
         tc::fence_after();
         const uint32_t ad = d0 + 12 * (it & 2) + 4 * (it & 1);
 #pragma unroll
@@ -932,7 +940,7 @@ __global__ void __launch_bounds__(cta_threads(SWAP), 1) shift_mma_kernel(const _
             bias[c] = P.bias != nullptr && col0 + c < P.cols ? __ldg(P.bias + col0 + c) : 0;
           __syncwarp();
         }
-        if (!wait(&bars->acc_full[b], (uint32_t)(seg_no / kAccBufs) & 1u, abort)) break;
+        if (!wait(&bars->acc_full[b], (uint32_t)(seg_no / kAccBufs) & 1u, bars)) break;
         tc::fence_after();
         for (int c0 = c_lo; c0 < c_hi; c0 += 16) {
           uint32_t rl[16], rh[16];
@@ -1154,7 +1162,7 @@ __global__ void __launch_bounds__(cta_threads(SWAP), 1) shift_mma_kernel(const _
 #pragma unroll
           for (int i = 0; i < 8; ++i) v[i] = pick_digit(v[i], (int)(now >> 1), digits);
         }
-        if (!wait(&bars->empty[slot], ring ^ 1u, abort)) break;
+        if (!wait(&bars->empty[slot], ring ^ 1u, bars)) break;
         const uint32_t dst = dst0 + slot * L::slot_bytes;
 #pragma unroll
         for (int i = 0; i < 8; ++i) {
@@ -1267,7 +1275,7 @@ __global__ void __launch_bounds__(cta_threads(SWAP), 1) shift_mma_kernel(const _
         const uint32_t la = lut_a + (bnd ? 0 : kLutBytes);
         // digit weights: [buffer][hi, lo, n3][16-index half][column][16 bytes]
         const uint32_t dd = dig0 + ((it >> 1) & 1) * 3 * L::digit_bytes + h * NL * 16;
-        if (!wait(&bars->empty[slot], ring ^ 1u, abort)) break;
+        if (!wait(&bars->empty[slot], ring ^ 1u, bars)) break;
 #pragma unroll
         for (int w8 = 0; w8 < kWords; ++w8) {
           const uint32_t nib = w8 ? cell.y : cell.x, b = (uint32_t)(16 * h + 8 * (kw + w8));
@@ -1304,7 +1312,7 @@ __global__ void __launch_bounds__(cta_threads(SWAP), 1) shift_mma_kernel(const _
       while (more) {
         const int b = seg_no % kAccBufs, n = w.c_end - w.chunk;
         const bool bounded = (w.fl & kBounded) != 0;
-        if (!wait(&bars->acc_empty[b], ((uint32_t)(seg_no / kAccBufs) & 1u) ^ 1u, abort)) break;
+        if (!wait(&bars->acc_empty[b], ((uint32_t)(seg_no / kAccBufs) & 1u) ^ 1u, bars)) break;
         tc::fence_after();
         const bool ok = kAccBufs == 1 || b == 0
                             ? issue_segment<N, PAIR, SWAP, 0>(bars, b0, d0, n, slot, ring, dbuf, bounded, pair_mask)
@@ -1322,13 +1330,21 @@ __global__ void __launch_bounds__(cta_threads(SWAP), 1) shift_mma_kernel(const _
     // rank of the cluster, or a convolution's last tile of the CTA): all warps
     // finish them, each rank its share of the columns.
     cg::cluster_group cl = cg::this_cluster();
+    cp_async_wait_all();  // none is in flight, unless this thread's role gave up
     tc::fence_before();
     if (split)
       cl.sync();
     else
       __syncthreads();
     tc::fence_after();
-    if (CONV || split) {
+    // A CTA that gave up has not made all of its sums: none of the CTAs whose sums
+    // meet then writes outputs from them, and no further pass runs (the places of its
+    // roles are lost).  Without a split the sums are the CTA's own, and its epilogue
+    // gave up if some are missing; the other CTA of the pair is looked at all the same.
+    int gone = 0;
+    if (CONV || split) gone = tc::ld_rank(tc::smem_u32(&bars->abort), min((uint32_t)lane, (uint32_t)(S.splits * kGroupSize - 1)));
+    const bool gave_up = __any_sync(0xffffffffu, gone != 0);
+    if ((CONV || split) && !gave_up) {
       Walk<kGroupSize, SWAP> v(S, flags, digits, split ? pass : -1);
       while (v.t + v.t_step < v.n_tiles) v.t += v.t_step;
       v.start_tile();
@@ -1438,11 +1454,14 @@ __global__ void __launch_bounds__(cta_threads(SWAP), 1) shift_mma_kernel(const _
       }
     }
     if (split) cl.sync();  // the peers' reads end before this shared memory changes
+    if (gave_up) break;
   }
 
   // every tensor operation has completed, in both CTAs of a pair, before tensor memory is freed
   __syncthreads();
-  if (CONV && tid == 0 && bars->amax && S.p[0].amax_out != nullptr) atomicMax(S.p[0].amax_out, bars->amax);
+  // a launch that gave up knows no bound of its incomplete outputs
+  const uint32_t cta_amax = bars->abort ? 0x80000000u : (CONV ? bars->amax : 0u);
+  if (tid == 0 && cta_amax && S.p[0].amax_out != nullptr) atomicMax(S.p[0].amax_out, cta_amax);
   if (warp == kMmaWarp) {
     if (cta == 0 && tc::elect_one()) tc::commit<PAIR>(&bars->done, pair_mask);
     __syncwarp();
@@ -1543,6 +1562,7 @@ template <int N, bool PAIR, bool SWAP = !PAIR>
 cudaError_t launch_set(const GemmParams* ps, int n, bool conv, cudaStream_t st) {
   MmaSet S{};
   S.n = n;
+  S.wait_cycles = g_wait_cycles.load(std::memory_order_relaxed);
   S.table_entries = 0;
   int64_t tiles = 0;
   int flag_off = 0;
@@ -1611,6 +1631,10 @@ cudaError_t launch_shift_mma(const GemmParams* ps, int n, bool conv, cudaStream_
   }
   if (!conv && rows <= kRows) return launch_set<64, false>(ps, n, false, st);  // few rows: swapped roles
   return cols <= 64 ? launch_set<64, true>(ps, n, conv, st) : launch_set<128, true>(ps, n, conv, st);
+}
+
+void set_mma_wait_cycles(long long cycles) {
+  g_wait_cycles.store(cycles > 0 ? cycles : kWaitCycles, std::memory_order_relaxed);
 }
 
 int read_mma_fault_flag() {

@@ -66,10 +66,15 @@ __device__ __forceinline__ void commit(uint64_t* bar, uint32_t cta_mask) {
                  : "memory");
 }
 
-// Cluster address of a shared-memory object of CTA rank, and an arrival there.
+// Cluster address of a shared-memory object of CTA rank, a load from it and an arrival there.
 __device__ __forceinline__ uint32_t map_rank(uint32_t addr, uint32_t rank) {
   uint32_t r;
   asm("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(addr), "r"(rank));
+  return r;
+}
+__device__ __forceinline__ int ld_rank(uint32_t addr, uint32_t rank) {
+  int r;
+  asm volatile("ld.shared::cluster.s32 %0, [%1];" : "=r"(r) : "r"(map_rank(addr, rank)) : "memory");
   return r;
 }
 __device__ __forceinline__ void mbar_arrive_cluster(uint32_t addr) {
