@@ -27,6 +27,11 @@ STATUS_NAMES = {0: "DS_OK", 1: "DS_ERR_INVALID_ARG", 2: "DS_ERR_SHAPE", 3: "DS_E
                 4: "DS_ERR_ALIGNMENT", 5: "DS_ERR_BUFFER_TOO_SMALL", 6: "DS_ERR_UNSUPPORTED",
                 7: "DS_ERR_CUDA"}
 
+# ds_linear_shift_route / ds_conv2d_shift_route
+DS_ROUTE_CUDA_CORES = 0
+DS_ROUTE_TENSOR_CORES = 1
+DS_ROUTE_TENSOR_CORES_SWAPPED = 2
+
 # flags
 DS_RELU = 1
 DS_AMAX_IN = 2
@@ -83,6 +88,8 @@ _SIGNATURES = {
     "ds_conv2d_shift": (ctypes.c_int, [ctypes.c_void_p, ctypes.POINTER(ds_weights), ctypes.c_void_p,
                                        ctypes.c_void_p, ctypes.c_void_p] + [ctypes.c_int] * 11 +
                         [ctypes.c_uint32, ctypes.c_void_p, ctypes.c_void_p]),
+    "ds_linear_shift_route": (ctypes.c_int, [ctypes.c_int64] * 3),
+    "ds_conv2d_shift_route": (ctypes.c_int, [ctypes.c_int] * 11),
     "ds_linear_shift_static_scratch": (ctypes.c_int, [ctypes.c_void_p, ctypes.POINTER(ds_weights),
                                                       ctypes.c_void_p, ctypes.c_void_p, ctypes.c_int64,
                                                       ctypes.c_int64, ctypes.c_int64, ctypes.c_uint32,
@@ -279,6 +286,15 @@ def ds_expand_shift_weights_bf16(w: ds_weights, buf, nbytes: int, stream=None) -
 
 def ds_linear_shift_bf16(x, w: ds_weights, bias, y, M: int, K: int, N: int, flags: int = 0, stream=None) -> None:
     _check(lib().ds_linear_shift_bf16(_ptr(x), ctypes.byref(w), _ptr(bias), _ptr(y), M, K, N, flags, _stream(stream)))
+
+
+def ds_linear_shift_route(M: int, K: int, N: int) -> int:
+    return int(lib().ds_linear_shift_route(M, K, N))
+
+
+def ds_conv2d_shift_route(N: int, C: int, H: int, W: int, K: int, R: int, S: int, stride_h: int, stride_w: int,
+                          pad_h: int, pad_w: int) -> int:
+    return int(lib().ds_conv2d_shift_route(N, C, H, W, K, R, S, stride_h, stride_w, pad_h, pad_w))
 
 
 def ds_bf16_fault_flag() -> int:

@@ -627,6 +627,40 @@ ds_status ds_linear_shift(const int32_t* x, const ds_weights* w, const int32_t* 
   return launch_fc(p, st);
 }
 
+int ds_linear_shift_route(int64_t M, int64_t K, int64_t N) {
+  clear_error();
+  if (M <= 0 || N <= 0 || M > (int64_t(1) << 40) || N > 65535LL * 64 || ds_packed_weight_bytes(N, K) == 0) return -1;
+  if (int32_tensor_bytes({M, K}) < 0 || int32_tensor_bytes({M, N}) < 0) return -1;
+  GemmParams p{};
+  p.rows = M;
+  p.kred = K;
+  p.cols = N;
+  p.n_chunks = blob_layout(N, K).n_chunks;
+  return shift_mma_route(&p, 1, false);
+}
+
+int ds_conv2d_shift_route(int N, int C, int H, int W, int K, int R, int S, int stride_h, int stride_w, int pad_h,
+                          int pad_w) {
+  clear_error();
+  int OH = 0, OW = 0;
+  if (N <= 0 || C <= 0 || K <= 0 ||
+      window_output(H, W, R, S, stride_h, stride_w, pad_h, pad_w, &OH, &OW) != DS_OK ||
+      check_image(C, H, W, OH, OW) != DS_OK || int32_tensor_bytes({N, C, H, W}) < 0 ||
+      int32_tensor_bytes({N, K, OH, OW}) < 0 || int32_tensor_bytes({C, R, S}) < 0 ||
+      ds_packed_weight_bytes(K, (int64_t)C * R * S) == 0)
+    return -1;
+  GemmParams p{};
+  p.rows = (int64_t)N * OH * OW;
+  p.kred = (int64_t)C * R * S;
+  p.cols = K;
+  p.n_chunks = blob_layout(K, p.kred).n_chunks;
+  p.H = H;
+  p.W = W;
+  p.R = R;
+  p.S = S;
+  return shift_mma_route(&p, 1, true);
+}
+
 ds_status ds_conv2d_shift(const int32_t* x, const ds_weights* w, const int32_t* bias,
                           const int32_t* residual, int32_t* y, int N, int C, int H, int W, int K,
                           int R, int S, int stride_h, int stride_w, int pad_h, int pad_w,

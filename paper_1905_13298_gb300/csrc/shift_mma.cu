@@ -49,10 +49,10 @@
 //   warps 16-21  operand B, three groups of two: decode the packed codes of a
 //                column through a table of weight bytes into shared memory
 //   warp 22      issues the tensor operations (swapped roles: warp 16, B after it)
-// FC layers of up to 128 rows swap the operands' roles: the lanes are 128 weight
-// columns, decoded into tensor memory, and N = 64 rows of x are expanded into
-// shared memory, so that no lane is idle and a code is decoded once per 64 rows
-// (VGG16 FC1 at batch 64: 0.361 ms with rows as lanes, 0.206 ms so, 0.189 ms now).
+// FC layers of up to 128 rows, and others of few tiles, swap the operands' roles: the
+// lanes are 128 weight columns, decoded into tensor memory, and N = 64 rows of x are
+// expanded into shared memory, so that no lane is idle and a code is decoded once per
+// 64 rows (VGG16 FC1 at batch 64: 0.361 ms with rows as lanes, 0.206 ms so, 0.189 ms now).
 // A ring of three slots of 16 reduction indices connects them; CTAs are
 // persistent over tiles and the ring runs on across them.  A grid that leaves
 // SMs idle splits the reduction over the CTAs of a cluster, which sum their
@@ -1594,42 +1594,59 @@ cudaError_t launch_set(const GemmParams* ps, int n, bool conv, cudaStream_t st) 
 
 }  // namespace
 
-// Rules of use, measured against the CUDA-core kernels.  A tile's fixed cost (its
-// epilogue, the ring's fill) is that of about 100 reduction indices: 1x1 layers of
-// 64 channels and 3x3 layers of 3 ran at 0.5-0.6 of the CUDA-core kernels' speed,
-// the 147 indices of a 7x7 layer of 3 channels at 1.2.  A launch's fixed cost (table,
-// tensor memory, cluster) is 3-4 us: FC of 64 x 2048 x 1000 (2^27 terms) ran at 1.2,
-// of 16 x 2048 x 1000 at 0.9; a convolution of 2^27 terms at 1.1.  Up to 8 rows an FC
-// layer is bound by its codes, which the cluster kernel reads once (8 x 25088 x
-// 4096: 0.94; 16 rows: 1.8).
-bool shift_mma_preferred(const GemmParams* ps, int n, bool conv) {
-  if (n < 1 || n > kMaxGemmPhases) return false;
+// Rules of use, measured against the CUDA-core kernels (us, CUDA cores -> here).  A
+// tile's fixed cost (its epilogue, the ring's fill) is that of about 100 reduction
+// indices: 1x1 layers of 64 channels and 3x3 layers of 3 ran at 0.5-0.6 of the
+// CUDA-core kernels' speed, the 147 indices of a 7x7 layer of 3 channels at 1.2.  A
+// launch's fixed cost (setup, ring fill, last tile, teardown) is about 10 us.
+// - Convolutions pay from 2^26 terms: 16x60x60 -> 32 3x3 34 -> 31, 512x23x23 -> 64 1x1
+//   37 -> 32, and none of the shapes tried there is slower by more than repeated runs
+//   differ (128x32x32 -> 128 1x1 28-31 -> 32).  The line at 1024 pixels is not a measured
+//   one: 16 images of 512x7x7 -> 512 3x3 (784 pixels) would take 100 for 212.
+// - FC pays from 2^27 terms (128 x 2048 x 512 43 -> 35) and 9 rows: up to 8 rows it is bound
+//   by its codes, which the cluster kernel reads once (8 x 25088 x 4096: 0.94; 16 rows: 1.8).
+// - Columns as lanes: up to 128 rows, as no lane is idle then.  With more rows, where
+//   the pairs' tiles are too few: a tile of 256 rows splits over 8 pairs at most, one of
+//   64 rows x 128 columns over 16 CTAs (1024 x 1028 x 128: pairs 56, so 31, CUDA cores 35;
+//   384 x 1368 x 256: 58, 29, 34).  The lines are at half of the pairs (38 tiles) and
+//   2^28.8 terms, from where a pair's wider tiles win (129 x 2036 x 4096: pairs 63, so 89), and
+//   for tiles of 64 columns, half of whose lanes would be idle, at 384 rows (384 x
+//   7724 x 64: pairs 55, so 37, CUDA cores 52; 1024 x 7725 x 48: 58, 99, 103).
+int shift_mma_route(const GemmParams* ps, int n, bool conv) {
+  if (n < 1 || n > kMaxGemmPhases) return DS_ROUTE_CUDA_CORES;
   int64_t tiles = 0, col_tiles = 0;
   double terms = 0.0;
   for (int i = 0; i < n; ++i) {
     const GemmParams& p = ps[i];
-    if (p.rows > INT32_MAX - kRows || p.n_chunks > INT32_MAX / kChunk) return false;
-    if (conv ? p.kred < 128 || p.rows < 1024 : p.rows <= 8) return false;
+    if (p.rows > INT32_MAX - kRows || p.n_chunks > INT32_MAX / kChunk) return DS_ROUTE_CUDA_CORES;
+    if (conv ? p.kred < 128 || p.rows < 1024 : p.rows <= 8) return DS_ROUTE_CUDA_CORES;
     terms += (double)p.rows * (double)p.kred * (double)p.cols;
     col_tiles += (p.cols + 63) / 64;
     tiles += (p.rows + kRows - 1) / kRows * ((p.cols + 63) / 64);
     if (conv) {
-      if (p.R > 16 || p.S > 15 || p.R * p.S > kMaxTaps) return false;
+      if (p.R > 16 || p.S > 15 || p.R * p.S > kMaxTaps) return DS_ROUTE_CUDA_CORES;
       // the tap tables' element offsets are 32-bit: 16 indices span up to 17 channels, the tables a few more
-      if ((int64_t)(kAGroups * kSlotK + 8) * p.H * p.W + (int64_t)p.R * p.W > INT32_MAX) return false;
+      if ((int64_t)(kAGroups * kSlotK + 8) * p.H * p.W + (int64_t)p.R * p.W > INT32_MAX) return DS_ROUTE_CUDA_CORES;
     }
   }
-  if (terms < (conv ? 67108864.0 : 134217728.0)) return false;
-  return col_tiles <= kMaxColTiles && tiles <= INT32_MAX / kMaxCluster;
+  if (terms < (conv ? 67108864.0 : 134217728.0)) return DS_ROUTE_CUDA_CORES;
+  if (col_tiles > kMaxColTiles || tiles > INT32_MAX / kMaxCluster) return DS_ROUTE_CUDA_CORES;
+  if (conv) return DS_ROUTE_TENSOR_CORES;
+  const int64_t rows = ps[0].rows, cols = ps[0].cols;
+  const bool swap = rows <= kRows ||
+                    (cols <= 64 ? rows <= 3 * kRows
+                                : (rows + 2 * kRows - 1) / (2 * kRows) * ((cols + 127) / 128) < 38 && terms < 469762048.0);
+  return swap ? DS_ROUTE_TENSOR_CORES_SWAPPED : DS_ROUTE_TENSOR_CORES;
+}
+
+bool shift_mma_preferred(const GemmParams* ps, int n, bool conv) {
+  return shift_mma_route(ps, n, conv) != DS_ROUTE_CUDA_CORES;
 }
 
 cudaError_t launch_shift_mma(const GemmParams* ps, int n, bool conv, cudaStream_t st) {
-  int64_t cols = 0, rows = 0;
-  for (int i = 0; i < n; ++i) {
-    cols = std::max(cols, ps[i].cols);
-    rows = std::max(rows, ps[i].rows);
-  }
-  if (!conv && rows <= kRows) return launch_set<64, false>(ps, n, false, st);  // few rows: swapped roles
+  if (shift_mma_route(ps, n, conv) == DS_ROUTE_TENSOR_CORES_SWAPPED) return launch_set<64, false>(ps, n, false, st);
+  int64_t cols = 0;
+  for (int i = 0; i < n; ++i) cols = std::max(cols, ps[i].cols);
   return cols <= 64 ? launch_set<64, true>(ps, n, conv, st) : launch_set<128, true>(ps, n, conv, st);
 }
 

@@ -1,0 +1,67 @@
+"""The size rules that choose a call's kernels, at sizes where both choices were timed (GB300, us per call).
+
+Each entry: the sizes, the route, and the times of the CUDA cores, the rows-as-lanes and the columns-as-lanes tensor-core
+kernels where they were taken.  The route must be the fastest of them, to 5%, or 1.5 us where all are short."""
+import pytest
+
+CC, TC, SWAP = 0, 1, 2
+FC = [
+    # M, K, N, route, CUDA cores, rows as lanes, columns as lanes
+    (8, 25088, 4096, CC, None, None, None),
+    (1024, 1028, 128, SWAP, 35.4, 56.4, 31.0),
+    (384, 1368, 256, SWAP, 33.5, 58.0, 29.0),
+    (256, 4100, 128, SWAP, 49.1, 64.2, 31.9),
+    (384, 5464, 64, SWAP, 41.4, 49.6, 33.1),
+    (384, 10924, 64, SWAP, 64.8, 61.9, 41.7),
+    (1024, 7725, 48, TC, 102.5, 57.8, 98.8),
+    (129, 2036, 4096, TC, 155.1, 62.5, 88.8),
+    (64, 25088, 4096, SWAP, 565.0, None, 189.0),
+    (8192, 4096, 4096, TC, 9930.0, 1460.0, None),
+]
+CONV = [
+    # N, C, H, W, K, R, stride, pad, route, CUDA cores, tensor cores
+    (4, 128, 32, 32, 128, 1, 1, 0, TC, 31.2, 32.1),
+    (5, 128, 39, 39, 128, 1, 1, 0, TC, 37.2, 33.0),
+    (5, 512, 23, 23, 64, 1, 1, 0, TC, 37.4, 31.6),
+    (5, 16, 60, 60, 32, 3, 1, 1, TC, 33.9, 30.7),
+    (32, 64, 56, 56, 64, 3, 1, 1, TC, 295.0, 109.0),
+    (32, 64, 56, 56, 64, 1, 1, 0, CC, None, None),
+]
+
+
+@pytest.fixture(scope="module")
+def ds():
+    from paper_1905_13298_gb300 import build
+    build.build_library()
+    import paper_1905_13298_gb300 as ds
+    ds.lib()
+    return ds
+
+
+def _fastest(times, route):
+    known = {i: t for i, t in enumerate(times) if t is not None}
+    assert not known or known[route] <= max(1.05 * min(known.values()), min(known.values()) + 1.5)
+
+
+@pytest.mark.parametrize("case", FC)
+def test_fc_route(ds, case):
+    M, K, N, route, *times = case
+    assert ds.ds_linear_shift_route(M, K, N) == route
+    _fastest(times, route)
+
+
+@pytest.mark.parametrize("case", CONV)
+def test_conv_route(ds, case):
+    B, C, H, W, K, R, st, pd, route, *times = case
+    assert ds.ds_conv2d_shift_route(B, C, H, W, K, R, R, st, st, pd, pd) == route
+    _fastest(times, route)
+
+
+def test_refused_sizes_have_no_route(ds):
+    assert ds.ds_linear_shift_route(0, 64, 64) == -1
+    assert ds.ds_linear_shift_route(64, 0, 64) == -1
+    assert ds.ds_linear_shift_route(64, 64, 65535 * 64 + 1) == -1
+    assert ds.ds_linear_shift_route(1 << 40, 1 << 40, 1) == -1
+    assert ds.ds_conv2d_shift_route(1, 64, 8, 8, 64, 9, 9, 1, 1, 0, 0) == -1  # kernel larger than the image
+    assert ds.ds_conv2d_shift_route(1, 64, 8, 8, 64, 3, 3, 0, 1, 0, 0) == -1
+    assert ds.ds_conv2d_shift_route(1, 1 << 20, 1 << 10, 1 << 10, 64, 1, 1, 1, 1, 0, 0) == -1
