@@ -35,8 +35,8 @@
 // sums are added between runs.  That is 19 tensor operations per 32 indices
 // instead of 17.  Inputs beyond 2^20 take one pass per 4-bit digit of x >> 16, the
 // lower digits unsigned.  The accumulator-width proof is the one of the other
-// integer kernels: where it fails, sums are 64-bit (half of the tile's columns at
-// a time) and saturated.
+// integer kernels: where it fails, sums are 64-bit (in tiles of 128 columns, half of
+// them at a time, in two walks: all of them have no room) and saturated.
 //
 // CTA: 128 rows (tensor-memory lanes) x N columns; a pair of CTAs shares a tile
 // of 256 rows, each decoding half of its weights (cta_group::2), since a tile's
@@ -159,7 +159,14 @@ struct Layout {
   static constexpr int NL = PAIR ? N / 2 : N;           // columns whose weights one CTA holds
   static constexpr int slot_bytes = kSlotK * NL * 16;
   static constexpr int digit_bytes = 2 * NL * 16;       // 32 indices, one operand
-  static constexpr int acc_bytes = N * kAccStride * 4;      // 32-bit sums, or 64-bit sums of half the columns
+  // 32-bit sums, or 64-bit sums of all columns where they have room (N = 64), else of half
+  // of them, in a second walk over the tile.  One walk instead of two, inputs up to 2^31
+  // (four digits), against the CUDA cores: 64x56x56 3x3 at batch 32 733 -> 395 us (567),
+  // 256x56x56 -> 64 1x1 400 -> 243 (318), the 7x7 stem 903 -> 566 (615), VGG16 FC1 at batch 64
+  // 1471 -> 754 (1169).  Tiles of 128 columns stay under them in two (1024x14x14 -> 256
+  // 1x1 484 against 592).
+  static constexpr bool halves = N > 64;
+  static constexpr int acc_bytes = N * kAccStride * (halves ? 4 : 8);
   static constexpr int xrow_bytes = kAWarps * 2 * 32 * kXStride * 4;
   __host__ __device__ static int base(int table_entries, int phases) {
     return (kTableOff + 2 * (4 * table_entries + 32) * 4 * phases + 1023) / 1024 * 1024;
@@ -190,7 +197,7 @@ __device__ __forceinline__ bool wait(uint64_t* bar, uint32_t parity, volatile Ba
 
 // The walk over a CTA's tiles, and in each tile over its segments (column half,
 // run, digit) and the 32-index chunks of a segment.  Every role walks alike.
-template <int GROUP, bool SWAP>
+template <int GROUP, bool SWAP, bool HALVES>
 struct Walk {
   const MmaSet& S;
   const uint8_t* flags;
@@ -237,8 +244,10 @@ struct Walk {
   __device__ __forceinline__ bool last_segment() const { return run == runs - 1 && d == digits - 1; }
   // Whether the last segment of the CTA's last tile (of its second half, if 64-bit) is being walked.
   __device__ __forceinline__ bool at_end() const {
-    return last_segment() && t + t_step >= n_tiles && ((fl & kInt32) || half == 1);
+    return last_segment() && t + t_step >= n_tiles && (one_walk() || half == 1);
   }
+  // Whether all columns are summed in one walk (HALVES: only 64-bit sums of half of the columns have room).
+  __device__ __forceinline__ bool one_walk() const { return !HALVES || (fl & kInt32); }
   // The place in the walk, kept in shared memory between a producer warp's
   // segments (its registers are needed in between); every lane has the same.
   static constexpr int kWords = 14;
@@ -258,7 +267,7 @@ struct Walk {
       d = 0;
       if (++run == runs) {
         run = 0;
-        if ((fl & kInt32) || split_half >= 0 || half == 1) {
+        if (one_walk() || split_half >= 0 || half == 1) {
           t += t_step;
           return false;
         }
@@ -270,8 +279,8 @@ struct Walk {
   }
 };
 
-template <int GROUP, bool SWAP>
-__device__ __forceinline__ bool next_segment_or_tile(Walk<GROUP, SWAP>& w) {
+template <int GROUP, bool SWAP, bool HALVES>
+__device__ __forceinline__ bool next_segment_or_tile(Walk<GROUP, SWAP, HALVES>& w) {
   if (w.next_segment()) return true;
   if (!w.valid()) return false;
   w.start_tile();
@@ -485,6 +494,7 @@ __device__ __forceinline__ bool issue_segment(Bars* bars, uint64_t b0, uint64_t 
 template <int N, bool PAIR, bool CONV, bool VEC, bool SWAP>
 __global__ void __launch_bounds__(cta_threads(SWAP), 1) shift_mma_kernel(const __grid_constant__ MmaSet S) {
   using L = Layout<N, PAIR>;
+  using Tiles = Walk<PAIR ? 2 : 1, SWAP, L::halves>;
   constexpr int NL = L::NL;            // columns whose weights this CTA decodes
   constexpr int kAccBufs = 128 / N;
   constexpr int kGroupSize = PAIR ? 2 : 1;
@@ -608,13 +618,13 @@ __global__ void __launch_bounds__(cta_threads(SWAP), 1) shift_mma_kernel(const _
       tc::mbar_arrive(bar);
   };
 
-  int* ws = reinterpret_cast<int*>(smem + kWalkOff) + warp * Walk<kGroupSize, SWAP>::kWords;
-  static_assert(kWalkOff + kThreads / 32 * Walk<kGroupSize, SWAP>::kWords * 4 <= kBiasOff, "one place per warp");
+  int* ws = reinterpret_cast<int*>(smem + kWalkOff) + warp * Tiles::kWords;
+  static_assert(kWalkOff + kThreads / 32 * Tiles::kWords * 4 <= kBiasOff, "one place per warp");
   const bool split = S.splits > 1;
-  // a split tile of 64-bit sums goes in two passes, one per half of the columns
+  // a split tile of 64-bit sums goes in two passes where a walk sums half of the columns
   int n_pass = 1;
-  if (split) {
-    Walk<kGroupSize, SWAP> w(S, flags, digits, 0);
+  if (L::halves && split) {
+    Tiles w(S, flags, digits, 0);
     w.start_tile();
     n_pass = (w.fl & kInt32) ? 1 : 2;
   }
@@ -638,7 +648,7 @@ __global__ void __launch_bounds__(cta_threads(SWAP), 1) shift_mma_kernel(const _
       int64_t cols = 0;
       const unsigned char *nsrc = nullptr, *bsrc = nullptr;
       auto seek = [&](bool first, int n) {
-        Walk<kGroupSize, SWAP> v(S, flags, digits, split ? pass : -1);
+        Tiles v(S, flags, digits, L::halves && split ? pass : -1);
         bool more = true;
         if (first) {
           v.start_tile();
@@ -755,7 +765,7 @@ __global__ void __launch_bounds__(cta_threads(SWAP), 1) shift_mma_kernel(const _
       const int32_t* tab = nullptr;
       // Moves n slots on, into later segments; false past the end of the sequence.
       auto seek = [&](bool first, int n) {
-        Walk<kGroupSize, SWAP> v(S, flags, digits, split ? pass : -1);
+        Tiles v(S, flags, digits, L::halves && split ? pass : -1);
         bool more = true;
         if (first) {
           v.start_tile();
@@ -916,7 +926,7 @@ __global__ void __launch_bounds__(cta_threads(SWAP), 1) shift_mma_kernel(const _
     } else if (warp < kFirstB) {
       // ---- epilogue: accumulators to integer sums in shared memory (which frees them for the next
       // segment), then from there, after the tile's last segment, to the output ----
-      Walk<kGroupSize, SWAP> w(S, flags, digits, split ? pass : -1);
+      Tiles w(S, flags, digits, L::halves && split ? pass : -1);
       w.start_tile();
       const int q = warp & 3, rowl = 32 * q + lane;
       int32_t* bias = reinterpret_cast<int32_t*>(smem + kBiasOff) + q * N;  // this warp's copy of the tile's biases
@@ -928,7 +938,7 @@ __global__ void __launch_bounds__(cta_threads(SWAP), 1) shift_mma_kernel(const _
         const bool i32 = (w.fl & kInt32) != 0, first = w.first_segment();
         // split tiles' sums, and a convolution's last ones, are left to all of the CTA's warps
         const bool out = w.last_segment() && !split && !(CONV && w.at_end());
-        const int c_lo = i32 ? 0 : w.half * (N / 2), c_hi = i32 ? N : c_lo + N / 2;
+        const int c_lo = !L::halves || i32 ? 0 : w.half * (N / 2), c_hi = !L::halves || i32 ? N : c_lo + N / 2;
         const int b = seg_no % kAccBufs, sh = 4 * w.d;
         const uint32_t acc = tmem + ((uint32_t)(32 * q) << 16) + b * 2 * N;
         // H holds 2^-17 of the digit sums, multiples of 2 (bounded tiles) or of 2^9
@@ -1092,7 +1102,7 @@ __global__ void __launch_bounds__(cta_threads(SWAP), 1) shift_mma_kernel(const _
       const int32_t* src = nullptr;
       bool in = false;
       auto seek = [&](bool first, int m) {
-        Walk<kGroupSize, SWAP> v(S, flags, digits, split ? pass : -1);
+        Tiles v(S, flags, digits, L::halves && split ? pass : -1);
         bool more = true;
         if (first) {
           v.start_tile();
@@ -1211,7 +1221,7 @@ __global__ void __launch_bounds__(cta_threads(SWAP), 1) shift_mma_kernel(const _
       int64_t cols = 0;
       const unsigned char *nsrc = nullptr, *bsrc = nullptr;
       auto seek = [&](bool first, int n) {
-        Walk<kGroupSize, SWAP> v(S, flags, digits, split ? pass : -1);
+        Tiles v(S, flags, digits, L::halves && split ? pass : -1);
         bool more = true;
         if (first) {
           v.start_tile();
@@ -1304,7 +1314,7 @@ __global__ void __launch_bounds__(cta_threads(SWAP), 1) shift_mma_kernel(const _
       }
     } else if (warp == kMmaWarp && cta == 0) {
       // ---- tensor operations (slot: chunks so far mod 3; it: digit buffer; ring: a bit per slot) ----
-      Walk<kGroupSize, SWAP> w(S, flags, digits, split ? pass : -1);
+      Tiles w(S, flags, digits, L::halves && split ? pass : -1);
       w.start_tile();
       const uint64_t b0 = tc::plain_desc(tc::smem_u32(bslots), NL * 16, 128);
       const uint64_t d0 = tc::plain_desc(tc::smem_u32(bdigits), NL * 16, 128);
@@ -1345,14 +1355,14 @@ __global__ void __launch_bounds__(cta_threads(SWAP), 1) shift_mma_kernel(const _
     if (CONV || split) gone = tc::ld_rank(tc::smem_u32(&bars->abort), min((uint32_t)lane, (uint32_t)(S.splits * kGroupSize - 1)));
     const bool gave_up = __any_sync(0xffffffffu, gone != 0);
     if ((CONV || split) && !gave_up) {
-      Walk<kGroupSize, SWAP> v(S, flags, digits, split ? pass : -1);
+      Tiles v(S, flags, digits, L::halves && split ? pass : -1);
       while (v.t + v.t_step < v.n_tiles) v.t += v.t_step;
       v.start_tile();
       const GemmParams& P = v.P();
       const bool i32 = (v.fl & kInt32) != 0;
-      const int per = (i32 ? N : N / 2) / S.splits, c_first = v.rank * per;
+      const int per = (!L::halves || i32 ? N : N / 2) / S.splits, c_first = v.rank * per;
       // the tile's accumulator columns are output columns, or rows with swapped roles
-      const int64_t col0 = (int64_t)v.ct * N + (i32 ? 0 : (split ? pass : 1) * (N / 2)) + c_first;
+      const int64_t col0 = (int64_t)v.ct * N + (!L::halves || i32 ? 0 : (split ? pass : 1) * (N / 2)) + c_first;
       const int64_t row0 = (int64_t)v.rt * (kRows * kGroupSize) + 128 * cta;
       const int nc = (int)min((int64_t)per, (SWAP ? P.rows : P.cols) - col0);
       const int32_t floor_v = (P.flags & DS_RELU) ? 0 : INT32_MIN;
