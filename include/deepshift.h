@@ -343,16 +343,17 @@ ds_status ds_linear_shift_static_scratch(const int32_t* x, const ds_weights* w, 
                                          int32_t* y, int64_t M, int64_t K, int64_t N, uint32_t flags,
                                          void* stream);
 
-/* Which kernels a call of these sizes runs, by the size rules alone (DS_CONV_IM2COL aside): DS_ROUTE_CUDA_CORES,
+/* Which kernels a call of these sizes runs, by the size rules alone (DS_CONV_IM2COL aside; amax_io: 0 for a call that
+ * passes NULL there): DS_ROUTE_CUDA_CORES,
  * DS_ROUTE_TENSOR_CORES (rows or pixels as the lanes) or DS_ROUTE_TENSOR_CORES_SWAPPED (output columns as the lanes);
  * -1 for sizes that the call refuses.  Results do not depend on it.  No device is needed.  A library utility: no
  * counterpart in the paper. */
 #define DS_ROUTE_CUDA_CORES 0
 #define DS_ROUTE_TENSOR_CORES 1
 #define DS_ROUTE_TENSOR_CORES_SWAPPED 2
-int ds_linear_shift_route(int64_t M, int64_t K, int64_t N);
+int ds_linear_shift_route(int64_t M, int64_t K, int64_t N, int amax_io);
 int ds_conv2d_shift_route(int N, int C, int H, int W, int K, int R, int S, int stride_h, int stride_w, int pad_h,
-                          int pad_w);
+                          int pad_w, int amax_io);
 
 /* ---------------------------------------------------------------------------
  * Chained forward (ResNet / VGG shaped networks of shift layers).

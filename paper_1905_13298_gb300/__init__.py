@@ -88,8 +88,8 @@ _SIGNATURES = {
     "ds_conv2d_shift": (ctypes.c_int, [ctypes.c_void_p, ctypes.POINTER(ds_weights), ctypes.c_void_p,
                                        ctypes.c_void_p, ctypes.c_void_p] + [ctypes.c_int] * 11 +
                         [ctypes.c_uint32, ctypes.c_void_p, ctypes.c_void_p]),
-    "ds_linear_shift_route": (ctypes.c_int, [ctypes.c_int64] * 3),
-    "ds_conv2d_shift_route": (ctypes.c_int, [ctypes.c_int] * 11),
+    "ds_linear_shift_route": (ctypes.c_int, [ctypes.c_int64] * 3 + [ctypes.c_int]),
+    "ds_conv2d_shift_route": (ctypes.c_int, [ctypes.c_int] * 12),
     "ds_linear_shift_static_scratch": (ctypes.c_int, [ctypes.c_void_p, ctypes.POINTER(ds_weights),
                                                       ctypes.c_void_p, ctypes.c_void_p, ctypes.c_int64,
                                                       ctypes.c_int64, ctypes.c_int64, ctypes.c_uint32,
@@ -288,13 +288,13 @@ def ds_linear_shift_bf16(x, w: ds_weights, bias, y, M: int, K: int, N: int, flag
     _check(lib().ds_linear_shift_bf16(_ptr(x), ctypes.byref(w), _ptr(bias), _ptr(y), M, K, N, flags, _stream(stream)))
 
 
-def ds_linear_shift_route(M: int, K: int, N: int) -> int:
-    return int(lib().ds_linear_shift_route(M, K, N))
+def ds_linear_shift_route(M: int, K: int, N: int, amax_io: bool = True) -> int:
+    return int(lib().ds_linear_shift_route(M, K, N, int(amax_io)))
 
 
 def ds_conv2d_shift_route(N: int, C: int, H: int, W: int, K: int, R: int, S: int, stride_h: int, stride_w: int,
-                          pad_h: int, pad_w: int) -> int:
-    return int(lib().ds_conv2d_shift_route(N, C, H, W, K, R, S, stride_h, stride_w, pad_h, pad_w))
+                          pad_h: int, pad_w: int, amax_io: bool = True) -> int:
+    return int(lib().ds_conv2d_shift_route(N, C, H, W, K, R, S, stride_h, stride_w, pad_h, pad_w, int(amax_io)))
 
 
 def ds_bf16_fault_flag() -> int:

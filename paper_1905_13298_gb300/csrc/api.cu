@@ -195,7 +195,8 @@ ds_status conv_launch(const int32_t* x, const ds_weights* w, const int32_t* bias
 }
 
 size_t conv_split_bytes(const GemmParams& p) {
-  if (shift_mma_preferred(&p, 1, true)) return 0;
+  // a chained forward's layers all have a bound on their input
+  if (shift_mma_route(&p, 1, true, true) != DS_ROUTE_CUDA_CORES) return 0;
   if (conv_pointwise_supported(p)) return conv_pointwise_split_bytes(p);
   return conv_direct_split_bytes(p);
 }
@@ -627,7 +628,7 @@ ds_status ds_linear_shift(const int32_t* x, const ds_weights* w, const int32_t* 
   return launch_fc(p, st);
 }
 
-int ds_linear_shift_route(int64_t M, int64_t K, int64_t N) {
+int ds_linear_shift_route(int64_t M, int64_t K, int64_t N, int amax_io) {
   clear_error();
   if (M <= 0 || N <= 0 || M > (int64_t(1) << 40) || N > 65535LL * 64 || ds_packed_weight_bytes(N, K) == 0) return -1;
   if (int32_tensor_bytes({M, K}) < 0 || int32_tensor_bytes({M, N}) < 0) return -1;
@@ -636,11 +637,11 @@ int ds_linear_shift_route(int64_t M, int64_t K, int64_t N) {
   p.kred = K;
   p.cols = N;
   p.n_chunks = blob_layout(N, K).n_chunks;
-  return shift_mma_route(&p, 1, false);
+  return shift_mma_route(&p, 1, false, amax_io != 0);
 }
 
 int ds_conv2d_shift_route(int N, int C, int H, int W, int K, int R, int S, int stride_h, int stride_w, int pad_h,
-                          int pad_w) {
+                          int pad_w, int amax_io) {
   clear_error();
   int OH = 0, OW = 0;
   if (N <= 0 || C <= 0 || K <= 0 ||
@@ -658,7 +659,7 @@ int ds_conv2d_shift_route(int N, int C, int H, int W, int K, int R, int S, int s
   p.W = W;
   p.R = R;
   p.S = S;
-  return shift_mma_route(&p, 1, true);
+  return shift_mma_route(&p, 1, true, amax_io != 0);
 }
 
 ds_status ds_conv2d_shift(const int32_t* x, const ds_weights* w, const int32_t* bias,

@@ -134,7 +134,7 @@ cudaError_t launch_conv2d_shift_phases(const GemmParams* ps, int n, cudaStream_t
 bool conv_narrow_supported(const GemmParams& p);
 cudaError_t launch_conv_narrow(const GemmParams& p, cudaStream_t st);
 // Defined in shift_mma.cu: exact shift sums on the tensor cores, up to kMaxGemmPhases GEMMs per launch.
-int shift_mma_route(const GemmParams* ps, int n, bool conv);  // DS_ROUTE_*
+int shift_mma_route(const GemmParams* ps, int n, bool conv, bool bound);  // DS_ROUTE_*; bound: max|x| is known
 bool shift_mma_preferred(const GemmParams* ps, int n, bool conv);
 cudaError_t launch_shift_mma(const GemmParams* ps, int n, bool conv, cudaStream_t st);
 int read_mma_fault_flag();

@@ -1615,6 +1615,17 @@ cudaError_t launch_set(const GemmParams* ps, int n, bool conv, cudaStream_t st) 
 //   one: 16 images of 512x7x7 -> 512 3x3 (784 pixels) would take 100 for 212.
 // - FC pays from 2^27 terms (128 x 2048 x 512 43 -> 35) and 9 rows: up to 8 rows it is bound
 //   by its codes, which the cluster kernel reads once (8 x 25088 x 4096: 0.94; 16 rows: 1.8).
+// - Without a bound on x (no amax_io) a call needs four digits and 64-bit sums: four
+//   walks in tiles of 64 columns or of swapped roles, eight in those of 128 columns.
+//   Convolutions take the first then (512x28x28 -> 512 1x1 at 4 images 101 -> 50, CUDA cores
+//   84), FC the second up to 64 pair tiles (384 x 10924 x 128 320 -> 100, CUDA cores 177; beyond,
+//   384 x 684 x 4096 169 -> 181).  The CUDA cores keep FC of up to 32 rows, where the cluster
+//   kernel has small tiles (VGG16 FC1 at 16 rows 539 -> 744, at 64 rows 1162 -> 747), FC of
+//   less than 128 indices (1024 x 68 x 4096 82 -> 94), and convolutions of 16 columns, less
+//   than 192 indices and 2^27.5 terms or more (16x171x171 -> 16 3x3 at 4 images 125 ->
+//   165; of 2^26 terms, 16x88x88 at 5 images, 103 -> 60).
+//   With amax_io the digits are known on the device only: VGG16 FC1 at 16 rows takes 337 ->
+//   188 up to 2^20, 337 -> 387 up to 2^24, 547 -> 570 up to 2^28 and 547 -> 751 beyond.
 // - Columns as lanes: up to 128 rows, as no lane is idle then.  With more rows, where
 //   the pairs' tiles are too few: a tile of 256 rows splits over 8 pairs at most, one of
 //   64 rows x 128 columns over 16 CTAs (1024 x 1028 x 128: pairs 56, so 31, CUDA cores 35;
@@ -1622,14 +1633,17 @@ cudaError_t launch_set(const GemmParams* ps, int n, bool conv, cudaStream_t st) 
 //   2^28.8 terms, from where a pair's wider tiles win (129 x 2036 x 4096: pairs 63, so 89), and
 //   for tiles of 64 columns, half of whose lanes would be idle, at 384 rows (384 x
 //   7724 x 64: pairs 55, so 37, CUDA cores 52; 1024 x 7725 x 48: 58, 99, 103).
-int shift_mma_route(const GemmParams* ps, int n, bool conv) {
+int shift_mma_route(const GemmParams* ps, int n, bool conv, bool bound) {
   if (n < 1 || n > kMaxGemmPhases) return DS_ROUTE_CUDA_CORES;
   int64_t tiles = 0, col_tiles = 0;
   double terms = 0.0;
+  bool few_columns = true;
   for (int i = 0; i < n; ++i) {
     const GemmParams& p = ps[i];
     if (p.rows > INT32_MAX - kRows || p.n_chunks > INT32_MAX / kChunk) return DS_ROUTE_CUDA_CORES;
     if (conv ? p.kred < 128 || p.rows < 1024 : p.rows <= 8) return DS_ROUTE_CUDA_CORES;
+    if (!bound && !conv && (p.kred < 128 || p.rows <= 32)) return DS_ROUTE_CUDA_CORES;
+    few_columns = few_columns && p.cols <= 16 && p.kred < 192 && p.R * p.S > 1;
     terms += (double)p.rows * (double)p.kred * (double)p.cols;
     col_tiles += (p.cols + 63) / 64;
     tiles += (p.rows + kRows - 1) / kRows * ((p.cols + 63) / 64);
@@ -1641,23 +1655,24 @@ int shift_mma_route(const GemmParams* ps, int n, bool conv) {
   }
   if (terms < (conv ? 67108864.0 : 134217728.0)) return DS_ROUTE_CUDA_CORES;
   if (col_tiles > kMaxColTiles || tiles > INT32_MAX / kMaxCluster) return DS_ROUTE_CUDA_CORES;
-  if (conv) return DS_ROUTE_TENSOR_CORES;
+  if (conv) return !bound && few_columns && terms >= 189812531.0 ? DS_ROUTE_CUDA_CORES : DS_ROUTE_TENSOR_CORES;
   const int64_t rows = ps[0].rows, cols = ps[0].cols;
-  const bool swap = rows <= kRows ||
-                    (cols <= 64 ? rows <= 3 * kRows
-                                : (rows + 2 * kRows - 1) / (2 * kRows) * ((cols + 127) / 128) < 38 && terms < 469762048.0);
+  const int64_t pair_tiles = (rows + 2 * kRows - 1) / (2 * kRows) * ((cols + 127) / 128);
+  const bool swap = rows <= kRows || (cols <= 64 ? rows <= 3 * kRows
+                                                 : (bound ? pair_tiles < 38 && terms < 469762048.0 : pair_tiles < 64));
   return swap ? DS_ROUTE_TENSOR_CORES_SWAPPED : DS_ROUTE_TENSOR_CORES;
 }
 
 bool shift_mma_preferred(const GemmParams* ps, int n, bool conv) {
-  return shift_mma_route(ps, n, conv) != DS_ROUTE_CUDA_CORES;
+  return shift_mma_route(ps, n, conv, ps[0].amax_in != nullptr) != DS_ROUTE_CUDA_CORES;
 }
 
 cudaError_t launch_shift_mma(const GemmParams* ps, int n, bool conv, cudaStream_t st) {
-  if (shift_mma_route(ps, n, conv) == DS_ROUTE_TENSOR_CORES_SWAPPED) return launch_set<64, false>(ps, n, false, st);
+  const bool bound = ps[0].amax_in != nullptr;
+  if (shift_mma_route(ps, n, conv, bound) == DS_ROUTE_TENSOR_CORES_SWAPPED) return launch_set<64, false>(ps, n, false, st);
   int64_t cols = 0;
   for (int i = 0; i < n; ++i) cols = std::max(cols, ps[i].cols);
-  return cols <= 64 ? launch_set<64, true>(ps, n, conv, st) : launch_set<128, true>(ps, n, conv, st);
+  return cols <= 64 || (conv && !bound) ? launch_set<64, true>(ps, n, conv, st) : launch_set<128, true>(ps, n, conv, st);
 }
 
 void set_mma_wait_cycles(long long cycles) {

@@ -183,3 +183,39 @@ def test_conv_stays_inside_its_buffers(dslib, geom):
 
     want = _finish(_sum(xp, s, p, product).reshape(B, OH, OW, K).permute(0, 3, 1, 2), 0.0, res)
     assert torch.equal(yg.view.reshape(res.shape), want)
+
+
+@pytest.mark.parametrize("shape", [(33, 4100, 1030, SWAP), (300, 8300, 500, SWAP), (2600, 1030, 1000, TC)])
+def test_fc_without_a_bound(dslib, shape):
+    """amax_io = NULL: four digits and 64-bit sums, whatever the values."""
+    ds, (M, K, N, route) = dslib, shape
+    assert ds.ds_linear_shift_route(M, K, N, False) == route
+    g = _gen(M)
+    s, p = _codes(g, (N, K), "uniform")
+    x, b = _values(g, (M, K), 1 << 31), torch.randint(-(1 << 16), 1 << 16, (N,), device="cuda", generator=g, dtype=torch.int32)
+    assert torch.equal(ds.linear_shift(x, ds.pack_shift_weights(s, p), b), _fc_want(x, s, p, b))
+
+
+@pytest.mark.parametrize("geom", [(8, 256, 14, 300, 3, 1), (4, 130, 41, 513, 1, 0), (3, 64, 40, 65, 3, 1)])
+def test_conv_without_a_bound(dslib, geom):
+    """The same for convolutions (tiles of 64 columns, more of them than 128-column ones) and their gradient."""
+    ds, (B, C, H, K, R, pd) = dslib, geom
+    assert ds.ds_conv2d_shift_route(B, C, H, H, K, R, R, 1, 1, pd, pd, False) == TC
+    g = _gen(sum(geom))
+    s, p = _codes(g, (K, C, R, R), "uniform")
+    x = _values(g, (B, C, H, H), 1 << 31)
+    y = ds.conv2d_shift(x, ds.pack_shift_weights(s, p), (R, R), None, (1, 1), (pd, pd))
+    xp = torch.nn.functional.pad(x, (pd,) * 4)
+
+    def product(a, w):
+        cols = a.unfold(2, R, 1).unfold(3, R, 1).permute(0, 2, 3, 1, 4, 5).reshape(B * H * H, C * R * R)
+        return cols @ w.reshape(K, -1).t()
+
+    assert torch.equal(y, _finish(_sum(xp, s, p, product).reshape(B, H, H, K).permute(0, 3, 1, 2), 0.0))
+    w = ds.pack_shift_weights_backward(s, p, (1, 1))
+    got = []
+    for flags in (0, ds.DS_CONV_IM2COL):
+        dx = torch.full((B, C, H, H), 7, dtype=torch.int32, device="cuda")
+        ds.ds_conv2d_shift_backward_x(y, w.desc, dx, B, C, H, H, K, R, R, 1, 1, pd, pd, flags, None)
+        got.append(dx)
+    assert torch.equal(*got)

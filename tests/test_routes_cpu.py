@@ -50,10 +50,48 @@ def test_fc_route(ds, case):
     _fastest(times, route)
 
 
+# the same without amax_io: M, K, N, route, CUDA cores, rows as lanes, columns as lanes
+FC_NO_BOUND = [
+    (16, 25088, 4096, CC, 538.9, None, 744.3),
+    (9, 25088, 4096, CC, 539.0, None, 744.2),
+    (64, 25088, 4096, SWAP, 1162.1, None, 747.6),
+    (128, 4096, 4096, SWAP, 417.6, None, 248.6),
+    (64, 4096, 1000, SWAP, 96.9, None, 82.1),
+    (384, 10924, 128, SWAP, 177.5, 319.8, 100.0),
+    (1024, 2052, 512, SWAP, 219.0, 249.0, 140.0),
+    (384, 684, 4096, TC, 226.0, 169.0, 181.0),
+    (1024, 68, 4096, CC, 82.0, None, 94.0),
+    (1024, 4096, 4096, TC, 2955.3, 1594.7, None),
+]
+CONV_NO_BOUND = [
+    # N, C, H, W, K, R, stride, pad, route, CUDA cores, tensor cores in tiles of 64 columns
+    (4, 16, 171, 171, 16, 3, 1, 1, CC, 124.9, 164.6),
+    (5, 16, 88, 88, 16, 3, 1, 1, TC, 103.0, 60.5),
+    (5, 128, 181, 181, 16, 1, 1, 0, TC, 243.0, 191.8),
+    (4, 128, 17, 17, 512, 1, 1, 0, TC, 45.6, 37.0),
+    (4, 512, 32, 32, 128, 1, 1, 0, TC, 83.0, 50.0),
+    (32, 64, 56, 56, 64, 3, 1, 1, TC, 559.0, 388.8),
+]
+
+
+@pytest.mark.parametrize("case", FC_NO_BOUND)
+def test_fc_route_without_a_bound(ds, case):
+    M, K, N, route, *times = case
+    assert ds.ds_linear_shift_route(M, K, N, False) == route
+    _fastest(times, route)
+
+
 @pytest.mark.parametrize("case", CONV)
 def test_conv_route(ds, case):
     B, C, H, W, K, R, st, pd, route, *times = case
     assert ds.ds_conv2d_shift_route(B, C, H, W, K, R, R, st, st, pd, pd) == route
+    _fastest(times, route)
+
+
+@pytest.mark.parametrize("case", CONV_NO_BOUND)
+def test_conv_route_without_a_bound(ds, case):
+    B, C, H, W, K, R, st, pd, route, *times = case
+    assert ds.ds_conv2d_shift_route(B, C, H, W, K, R, R, st, st, pd, pd, False) == route
     _fastest(times, route)
 
 
