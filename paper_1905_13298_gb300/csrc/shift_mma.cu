@@ -1621,9 +1621,10 @@ cudaError_t launch_set(const GemmParams* ps, int n, bool conv, cudaStream_t st) 
 //   84), FC the second up to 64 pair tiles (384 x 10924 x 128 320 -> 100, CUDA cores 177; beyond,
 //   384 x 684 x 4096 169 -> 181).  The CUDA cores keep FC of up to 32 rows, where the cluster
 //   kernel has small tiles (VGG16 FC1 at 16 rows 539 -> 744, at 64 rows 1162 -> 747), FC of
-//   less than 128 indices (1024 x 68 x 4096 82 -> 94), and convolutions of 16 columns, less
-//   than 192 indices and 2^27.5 terms or more (16x171x171 -> 16 3x3 at 4 images 125 ->
-//   165; of 2^26 terms, 16x88x88 at 5 images, 103 -> 60).
+//   less than 128 indices (1024 x 68 x 4096 82 -> 94), and convolutions of 16 columns and
+//   less than 192 indices from 2^27 terms (16x121x121 -> 16 3x3 at 4 images 68 -> 101; of
+//   2^26 terms, 16x88x88 at 5 images, 103 -> 60), kernels beyond 3x3 from 2^27.5 (3x119x119 -> 16
+//   7x7 at 5 images 189 -> 104, 3x169x169 at 4 images 121 -> 147).
 //   With amax_io the digits are known on the device only: VGG16 FC1 at 16 rows takes 337 ->
 //   188 up to 2^20, 337 -> 387 up to 2^24, 547 -> 570 up to 2^28 and 547 -> 751 beyond.
 // - Columns as lanes: up to 128 rows, as no lane is idle then.  With more rows, where
@@ -1655,7 +1656,8 @@ int shift_mma_route(const GemmParams* ps, int n, bool conv, bool bound) {
   }
   if (terms < (conv ? 67108864.0 : 134217728.0)) return DS_ROUTE_CUDA_CORES;
   if (col_tiles > kMaxColTiles || tiles > INT32_MAX / kMaxCluster) return DS_ROUTE_CUDA_CORES;
-  if (conv) return !bound && few_columns && terms >= 189812531.0 ? DS_ROUTE_CUDA_CORES : DS_ROUTE_TENSOR_CORES;
+  if (conv && !bound && few_columns && terms >= (ps[0].R * ps[0].S <= 9 ? 134217728.0 : 189812531.0)) return DS_ROUTE_CUDA_CORES;
+  if (conv) return DS_ROUTE_TENSOR_CORES;
   const int64_t rows = ps[0].rows, cols = ps[0].cols;
   const int64_t pair_tiles = (rows + 2 * kRows - 1) / (2 * kRows) * ((cols + 127) / 128);
   const bool swap = rows <= kRows || (cols <= 64 ? rows <= 3 * kRows

@@ -67,6 +67,9 @@ CONV_NO_BOUND = [
     # N, C, H, W, K, R, stride, pad, route, CUDA cores, tensor cores in tiles of 64 columns
     (4, 16, 171, 171, 16, 3, 1, 1, CC, 124.9, 164.6),
     (5, 16, 88, 88, 16, 3, 1, 1, TC, 103.0, 60.5),
+    (4, 16, 121, 121, 16, 3, 1, 1, CC, 67.9, 100.7),
+    (5, 3, 119, 119, 16, 7, 1, 3, TC, 188.8, 103.9),
+    (4, 3, 169, 169, 16, 7, 1, 3, CC, 121.2, 147.0),
     (5, 128, 181, 181, 16, 1, 1, 0, TC, 243.0, 191.8),
     (4, 128, 17, 17, 512, 1, 1, 0, TC, 45.6, 37.0),
     (4, 512, 32, 32, 128, 1, 1, 0, TC, 83.0, 50.0),
