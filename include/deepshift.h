@@ -79,7 +79,7 @@ size_t ds_abi_struct_size(int which);
  * Flags of the compute calls
  * ------------------------------------------------------------------------- */
 #define DS_RELU 1u      /* y = max(y, 0) after saturation (and after the residual add) */
-#define DS_AMAX_IN 2u   /* amax_io[0] already holds max|x| of the input: skip the pre-pass */
+#define DS_AMAX_IN 2u   /* amax_io[0] already holds max|x| of the input, or more: skip the pre-pass */
 #define DS_AMAX_OUT 4u  /* write max|y| over this call's outputs into amax_io[1] */
 #define DS_RESIDUAL 8u  /* conv only: y = sat32(sat32(conv) + residual) before the ReLU */
 #define DS_FORCE_INT64 16u /* always use the 64-bit accumulator path (testing / worst case) */
@@ -284,6 +284,13 @@ void ds_bf16_set_wait_limit(long long cycles);
  * set, else from a pre-pass over x that writes it to amax_io[0].  amax_io
  * (device, 2 x u32) may be NULL: then no bound is available and the 64-bit
  * path is always taken (DS_AMAX_IN and DS_AMAX_OUT need amax_io).
+ *
+ * amax also says how much of x the tensor-core kernels read: up to 2^20 they
+ * take 20 bits and a sign, up to 2^24, 2^28 and beyond 4 bits more each (and a
+ * pass over x each).  So a word of DS_AMAX_IN must be at least max|x|: one that
+ * is larger costs time, one that is smaller gives wrong results even where the
+ * sums would fit.  Nothing may change the word while the call runs: calls that
+ * can overlap on the GPU each need words of their own.
  * ------------------------------------------------------------------------- */
 
 /*

@@ -41,7 +41,7 @@
 // CTA: 128 rows (tensor-memory lanes) x N columns; a pair of CTAs shares a tile
 // of 256 rows, each decoding half of its weights (cta_group::2), since a tile's
 // weight bytes are written to and read from shared memory once per 128 or 256
-// rows.  23 warps (swapped roles, below: 25), with x as operand A:
+// rows.  23 warps (swapped roles, below: 27, two of them idle), with x as operand A:
 //   warps 0-11   operand A, three groups of four: a thread gathers 16 values of
 //                its row, expands them and writes them to tensor memory
 //   warps 12-15  epilogue: accumulators to integer sums in shared memory, then
@@ -98,7 +98,7 @@ static_assert(kAGroups == kSlots, "a group of operand-A warps per ring slot");
 // warps 0-11 operand A, 12-15 epilogue, then operand B, then the tensor operations
 constexpr int kFirstEpi = kAWarps, kFirstB = kFirstEpi + kEpiWarps;
 // Operand B: three groups of two warps, or with swapped roles two of four.  23
-// warps leave a thread 80 registers, 25 leave 72: with 72 the convolution's operand
+// warps leave a thread 80 registers, from 25 on it is 72: with 72 the convolution's operand
 // A spills in its loop (a version with 270 spilled bytes ran 15-30% slower).
 __host__ __device__ constexpr int b_warps(bool swap) { return swap ? 8 : 6; }
 __device__ __forceinline__ int swapped_b_warp(int warp) {
@@ -106,9 +106,7 @@ __device__ __forceinline__ int swapped_b_warp(int warp) {
 }
 // Swapped roles: the issuing warp is warp 16 and B's are 17-19, 21-23, 25 and 26 (20
 // and 24 idle), so that no B warp is on its scheduler: VGG16 FC1 at batch 64 0.205
-// -> 0.193 ms on one GPU in turn.  The unswapped kernels' roles are as before, but their
-// convolutions measured 3-6% faster with the changed branch conditions (64x56x56 3x3
-// 0.125 -> 0.117 ms, FC unchanged); why was not isolated.  (Unswapped, the two more warps would cost the 80 registers.)
+// -> 0.193 ms on one GPU in turn.  (Unswapped, two more warps would cost the 80 registers.)
 __host__ __device__ constexpr int cta_threads(bool swap) { return 32 * (swap ? 27 : kFirstB + b_warps(false) + 1); }
 constexpr int kCodeAhead = 4;   // slots of a B group whose codes are in flight
 constexpr int kCodeBytes = kCodeAhead * b_warps(false) * 32 * 16;
@@ -611,7 +609,15 @@ __global__ void __launch_bounds__(cta_threads(SWAP), 1) shift_mma_kernel(const _
     __syncthreads();
   tc::fence_after();
   constexpr uint32_t tmem = 0;  // all 512 columns are this CTA's, so they start at column 0
-  auto arrive = [&](uint64_t* bar) {  // at the CTA that issues the tensor operations
+  // Arrivals at the barriers of the CTA that issues the tensor operations.  From the
+  // other CTA of a pair they publish writes to that CTA's own shared and tensor memory,
+  // which no thread of the issuing CTA reads: each SM's tensor unit reads its own
+  // CTA's operands, and before its arrival a warp has waited for its tensor-memory
+  // stores and fenced its shared-memory writes for the asynchronous proxy.  So the
+  // instruction's default ordering (release at CTA scope) is left as it is; release
+  // at cluster scope measured 830-1190 clocks an arrival instead of 5-15, FC of 4096 rows
+  // 1766 us instead of 1150.
+  auto arrive = [&](uint64_t* bar) {
     if constexpr (PAIR)
       tc::mbar_arrive_cluster(tc::map_rank(tc::smem_u32(bar), leader));
     else
