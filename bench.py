@@ -140,6 +140,11 @@ def tensor_peak(dev=None):
     return tops * TENSOR_INT_OPS_PER_CLK_PER_SM / INT_OPS_PER_CLK_PER_SM, sms, sm_max, kind
 
 
+def route_peak(dev, route: int):
+    """(name, T int-op equivalents/s) of the roofline of the kernels that a call's sizes select (ds_*_route)."""
+    return ("tensor", tensor_peak(dev)[0]) if route > 0 else ("alu", alu_peak(dev)[0])
+
+
 def smi_gpu_id(index: int, visible: str | None) -> str:
     """nvidia-smi's --id of this process's CUDA device `index`: CUDA numbers only the devices listed in
     CUDA_VISIBLE_DEVICES (indices or UUIDs, both accepted by --id), nvidia-smi every GPU of the machine."""
@@ -364,7 +369,6 @@ def run_gpu_other(args, wl, rank, world, local_rank):
     clocks = sampler.stop()
     ms = e0.elapsed_time(e1)
     peaks, _ = measured_peaks()
-    alu_tops = tensor_peak(dev)[0]
     value = terms * args.steps / (ms / 1e3) / 1e9
     if wl["kind"] == "fc16":
         tflops = 2 * terms / (ms / args.steps / 1e3) / 1e12
@@ -372,7 +376,10 @@ def run_gpu_other(args, wl, rank, world, local_rank):
         roof = {"bound": "tensor", "achieved": tflops, "peak": peak, "unit": "TFLOP/s", "frac": tflops / peak,
                 "traffic": None, "kernel": "linear_bf16_kernel", "peak_basis": "bf16_tflops (burst), measured"}
     else:
-        roof = {"bound": "tensor", "achieved": 2 * terms / (ms / args.steps / 1e3) / 1e12, "peak": alu_tops,
+        # a network's layers run on both kinds of kernels: its fraction is of the faster kind's roofline
+        bound, alu_tops = route_peak(dev, ds.ds_linear_shift_route(wl["M"], wl["K"], wl["Nout"])
+                                     if wl["kind"] == "fc" else ds.DS_ROUTE_TENSOR_CORES)
+        roof = {"bound": bound, "achieved": 2 * terms / (ms / args.steps / 1e3) / 1e12, "peak": alu_tops,
                 "unit": "Tintop/s", "frac": 2 * terms / (ms / args.steps / 1e3) / 1e12 / alu_tops,
                 "traffic": None, "kernel": "whole step"}
     out = {"metric": METRIC, "value": value, "unit": METRIC, "n_gpus": 1, "steps": args.steps, "warmup": args.warmup,
@@ -492,8 +499,9 @@ def time_fc_layer(args, ds, dev, seed, M, K, N, backward=False):
     torch.cuda.synchronize()
     ms = e0.elapsed_time(e1) / reps
     terms = M * K * N
-    return dict(shape=f"FC {K}->{N}", terms=terms, ms=ms, gsops=terms / ms / 1e6,
-                frac=2 * terms / (ms / 1e3) / (tensor_peak(dev)[0] * 1e12))
+    bound, tops = route_peak(dev, ds.ds_linear_shift_route(*((M, N, K) if backward else (M, K, N))))
+    return dict(shape=f"FC {K}->{N}", terms=terms, ms=ms, gsops=terms / ms / 1e6, bound=bound,
+                frac=2 * terms / (ms / 1e3) / (tops * 1e12))
 
 
 def run_specialized(args, wl, local_rank):
@@ -634,8 +642,15 @@ def run_layer_sweep(args, wl, local_rank):
         torch.cuda.synchronize()
         ms = e0.elapsed_time(e1) / reps
         terms = B * sp.K * OH * OW * sp.C * sp.R * sp.S
+        if not bwd:
+            route = ds.ds_conv2d_shift_route(B, sp.C, sp.H, sp.W, sp.K, sp.R, sp.S, sp.stride, sp.stride, sp.pad, sp.pad)
+        elif sp.stride == 1:  # the forward convolution of dY with the transposed codes
+            route = ds.ds_conv2d_shift_route(B, sp.K, OH, OW, sp.C, sp.R, sp.S, 1, 1, sp.R - 1 - sp.pad, sp.S - 1 - sp.pad)
+        else:  # a strided layer's gradient: tap phases, of either kind
+            route = ds.DS_ROUTE_TENSOR_CORES
+        bound, tops = route_peak(dev, route)
         r = dict(layer=i, shape=f"{sp.C}x{sp.H}x{sp.W}->{sp.K} {sp.R}x{sp.S}/{sp.stride}", terms=terms, ms=ms,
-                 gsops=terms / ms / 1e6, frac=2 * terms / (ms / 1e3) / (tensor_peak(dev)[0] * 1e12))
+                 gsops=terms / ms / 1e6, bound=bound, frac=2 * terms / (ms / 1e3) / (tops * 1e12))
         seen[key] = r
         rows.append(r)
         tot_terms += terms
