@@ -219,3 +219,68 @@ def test_conv_without_a_bound(dslib, geom):
         ds.ds_conv2d_shift_backward_x(y, w.desc, dx, B, C, H, H, K, R, R, 1, 1, pd, pd, flags, None)
         got.append(dx)
     assert torch.equal(*got)
+
+
+def _small_calls(ds, seed):
+    """One FC call (columns as lanes, split) and one convolution (pairs, split): closures over fresh tensors, and checks."""
+    g = _gen(seed)
+    s, p = _codes(g, (1030, 2052), "uniform")
+    x, b = _values(g, (64, 2052), 1 << 20), torch.randint(-(1 << 16), 1 << 16, (1030,), device="cuda", generator=g, dtype=torch.int32)
+    w, a = ds.pack_shift_weights(s, p), torch.zeros(2, dtype=torch.int32, device="cuda")
+    sc, pc = _codes(g, (130, 64, 3, 3), "centred")
+    xc = _values(g, (2, 64, 24, 24), 1 << 20)
+    wc, ac = ds.pack_shift_weights(sc, pc), torch.zeros(2, dtype=torch.int32, device="cuda")
+    y = torch.empty((64, 1030), dtype=torch.int32, device="cuda")
+    yc = torch.empty((2, 130, 24, 24), dtype=torch.int32, device="cuda")
+
+    def call(stream):
+        ds.ds_linear_shift(x, w.desc, b, y, 64, 2052, 1030, 0, a, stream)
+        ds.ds_conv2d_shift(xc, wc.desc, None, None, yc, 2, 64, 24, 24, 130, 3, 3, 1, 1, 1, 1, 0, ac, stream)
+
+    def check():
+        assert torch.equal(y, _fc_want(x, s, p, b))
+        cols = torch.nn.functional.pad(xc, (1,) * 4).unfold(2, 3, 1).unfold(3, 3, 1).permute(0, 2, 3, 1, 4, 5).reshape(1152, 576)
+        want = _finish(_sum(cols, sc.reshape(130, -1), pc.reshape(130, -1), lambda v, u: v @ u.t()), 0.0)
+        assert torch.equal(yc.permute(0, 2, 3, 1).reshape(1152, 130), want)
+
+    return call, check, (x, xc)
+
+
+def test_calls_on_two_threads_and_streams(dslib):
+    import threading
+    work = [_small_calls(dslib, seed) for seed in (3, 4)]
+    torch.cuda.synchronize()
+    errors = []
+
+    def go(call):
+        try:
+            stream = torch.cuda.Stream()
+            for _ in range(20):
+                call(stream.cuda_stream)
+            stream.synchronize()
+        except Exception as e:  # reported by the main thread
+            errors.append(e)
+
+    threads = [threading.Thread(target=go, args=(w[0],)) for w in work]
+    for t in threads:
+        t.start()
+    for t in threads:
+        t.join()
+    assert not errors, errors
+    for _, check, _ in work:
+        check()
+
+
+def test_captured_calls_follow_new_inputs(dslib):
+    call, check, inputs = _small_calls(dslib, 5)
+    call(torch.cuda.current_stream().cuda_stream)  # kernel attributes are set at the first launch
+    torch.cuda.synchronize()
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph):
+        call(torch.cuda.current_stream().cuda_stream)
+    for shift in (1, 2):
+        for t in inputs:
+            t.copy_(torch.roll(t, shift, 0) >> shift)
+        graph.replay()
+        torch.cuda.synchronize()
+        check()
