@@ -1636,10 +1636,13 @@ cudaError_t launch_set(const GemmParams* ps, int n, bool conv, cudaStream_t st) 
 // - Columns as lanes: up to 128 rows, as no lane is idle then.  With more rows, where
 //   the pairs' tiles are too few: a tile of 256 rows splits over 8 pairs at most, one of
 //   64 rows x 128 columns over 16 CTAs (1024 x 1028 x 128: pairs 56, so 31, CUDA cores 35;
-//   384 x 1368 x 256: 58, 29, 34).  The lines are at half of the pairs (38 tiles) and
-//   2^28.8 terms, from where a pair's wider tiles win (129 x 2036 x 4096: pairs 63, so 89), and
-//   for tiles of 64 columns, half of whose lanes would be idle, at 384 rows (384 x
-//   7724 x 64: pairs 55, so 37, CUDA cores 52; 1024 x 7725 x 48: 58, 99, 103).
+//   384 x 1368 x 256: 58, 29, 34; 384 x 10924 x 128: 81, 44, 98).  The lines are at half of
+//   the pairs (38 tiles) and 2^29.6 terms (2^29.2 where rows of x are copied word by word,
+//   2^28.8 where the small tiles fill half of the chip unsplit): from there on a pair's wider
+//   tiles win or come near (129 x 1021 x 4096: pairs 52, so 62; 1024 x 5797 x 128: 72, 80;
+//   1024 x 8196 x 128: 75, 89; 256 x 4196 x 1000 still 66, 51).  For tiles of 64 columns,
+//   half of whose lanes would be idle, the line is at 384 rows (384 x 7724 x 64: pairs
+//   55, so 37, CUDA cores 52; 1024 x 7725 x 48: 58, 99, 103).
 int shift_mma_route(const GemmParams* ps, int n, bool conv, bool bound) {
   if (n < 1 || n > kMaxGemmPhases) return DS_ROUTE_CUDA_CORES;
   int64_t tiles = 0, col_tiles = 0;
@@ -1666,8 +1669,12 @@ int shift_mma_route(const GemmParams* ps, int n, bool conv, bool bound) {
   if (conv) return DS_ROUTE_TENSOR_CORES;
   const int64_t rows = ps[0].rows, cols = ps[0].cols;
   const int64_t pair_tiles = (rows + 2 * kRows - 1) / (2 * kRows) * ((cols + 127) / 128);
+  const int64_t swap_tiles = (rows + 63) / 64 * ((cols + kRows - 1) / kRows);
   const bool swap = rows <= kRows || (cols <= 64 ? rows <= 3 * kRows
-                                                 : (bound ? pair_tiles < 38 && terms < 469762048.0 : pair_tiles < 64));
+                                      : !bound   ? pair_tiles < 64
+                                                 : pair_tiles < 38 && terms < (swap_tiles > 76         ? 469762048.0
+                                                                               : ps[0].kred % 4 != 0 ? 603979776.0
+                                                                                                     : 805306368.0));
   return swap ? DS_ROUTE_TENSOR_CORES_SWAPPED : DS_ROUTE_TENSOR_CORES;
 }
 

@@ -14,7 +14,7 @@ CANARY = 0x5A5A5A5A
 FC = [
     (64, 8192, 4096),    # columns as lanes, split
     (64, 512, 19500),    # columns as lanes, a tile a CTA
-    (256, 4096, 512),    # rows as lanes, split
+    (256, 8192, 512),    # rows as lanes, split
     (2560, 2048, 1024),  # rows as lanes, a tile a pair of CTAs
 ]
 CONV = [

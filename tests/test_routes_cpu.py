@@ -14,7 +14,14 @@ FC = [
     (384, 5464, 64, SWAP, 41.4, 49.6, 33.1),
     (384, 10924, 64, SWAP, 64.8, 61.9, 41.7),
     (1024, 7725, 48, TC, 102.5, 57.8, 98.8),
+    (384, 10924, 128, SWAP, 98.0, 81.0, 44.0),
+    (1024, 2900, 256, SWAP, 86.0, 60.0, 43.0),
+    (129, 1440, 4096, TC, 116.0, 55.0, 60.0),
     (129, 2036, 4096, TC, 155.1, 62.5, 88.8),
+    (129, 1021, 4096, TC, 92.8, 51.9, 61.5),
+    (1024, 5796, 128, SWAP, 91.0, 69.0, 62.0),
+    (1024, 5797, 128, TC, 98.6, 71.8, 80.1),
+    (1024, 8196, 128, TC, 124.0, 75.0, 89.0),
     (64, 25088, 4096, SWAP, 565.0, None, 189.0),
     (8192, 4096, 4096, TC, 9930.0, 1460.0, None),
 ]
