@@ -34,7 +34,7 @@ TENSOR_INT_OPS_PER_CLK_PER_SM = 2 * 8192 / 17
 ALG_INT_OPS_PER_TERM = 2      # one shift + one add/subtract per term (Fig. 1a: MAC -> shift + add)
 # DRAM bytes (read + write) of one shift_mma_kernel<64,1,1,0,0> launch on this workload, from one ncu capture
 # of the current kernel (dram__bytes_read.sum + dram__bytes_write.sum); y stays in L2 at kernel end.
-NCU_TRAFFIC_BYTES = 25.86e6
+NCU_TRAFFIC_BYTES = 26.43e6
 HBM_NOMINAL_GBS = 7900.0  # GB300 HBM3e, nominal
 E2E_CHUNKS = 4  # chunks of the batch in the end-to-end measurement
 

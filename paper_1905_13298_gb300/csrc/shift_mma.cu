@@ -52,7 +52,7 @@
 // FC layers of up to 128 rows, and others of few tiles, swap the operands' roles: the
 // lanes are 128 weight columns, decoded into tensor memory, and N = 64 rows of x are
 // expanded into shared memory, so that no lane is idle and a code is decoded once per
-// 64 rows (VGG16 FC1 at batch 64: 0.361 ms with rows as lanes, 0.206 ms so, 0.189 ms now).
+// 64 rows (VGG16 FC1 at batch 64: 0.361 ms with rows as lanes, 0.189 ms so).
 // A ring of three slots of 16 reduction indices connects them; CTAs are
 // persistent over tiles and the ring runs on across them.  A grid that leaves
 // SMs idle splits the reduction over the CTAs of a cluster, which sum their
@@ -61,11 +61,12 @@
 // its sums.  The cluster barriers need no bound of their own: every CTA reaches
 // them, since its roles' waits are bounded.
 //
-// Measured (GB300, per call with the max|x| pre-pass, against the CUDA-core
-// kernels): FC 8192 x 4096 x 4096 9.94 -> 1.46 ms (about 760 clocks a slot of 16
-// indices; the operations alone take 608), ConvShift 64x56x56 3x3 at batch 32 0.296
-// -> 0.112 ms, 256x14x14 -> 512 3x3/2 0.216 -> 0.051 ms, 1024x14x14 -> 256 1x1 at batch
-// 64 0.301 -> 0.086 ms, VGG16 FC1 at batch 64 0.565 -> 0.189 ms.  What bounds it: at
+// Measured (GB300, back to back over changing inputs, with the max|x| pre-pass,
+// CUDA-core kernels -> here): FC 8192 x 4096 x 4096 9.93 -> 1.53 ms (one input again and
+// again: 1.47; about 760 clocks a slot of 16 indices, of which the operations alone
+// take 608), ConvShift 64x56x56 3x3 at batch 32 with a residual 0.296 -> 0.110 ms,
+// 256x14x14 -> 512 3x3/2 0.216 -> 0.051 ms, 1024x14x14 -> 256 1x1 at batch 64 0.301 -> 0.086
+// ms, VGG16 FC1 at batch 64 0.565 -> 0.189 ms.  What bounds it: at
 // N = 128 the ALU pipe (expanding x: 5-6 of its instructions a value, which run
 // at 64 lanes a clock and SM) and the operations' issue; at N = 64 the issuing
 // warp (about 590 clocks a slot with nothing else done, against 272 of
