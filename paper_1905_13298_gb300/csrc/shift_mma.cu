@@ -1359,7 +1359,8 @@ __global__ void __launch_bounds__(cta_threads(SWAP), 1) shift_mma_kernel(const _
     // roles are lost).  Without a split the sums are the CTA's own, and its epilogue
     // gave up if some are missing; the other CTA of the pair is looked at all the same.
     int gone = 0;
-    if (CONV || split) gone = tc::ld_rank(tc::smem_u32(&bars->abort), min((uint32_t)lane, (uint32_t)(S.splits * kGroupSize - 1)));
+    if (CONV || split)
+      gone = tc::ld_rank(tc::smem_u32(&bars->abort), min((uint32_t)lane, (uint32_t)(S.splits * kGroupSize - 1)));
     const bool gave_up = __any_sync(0xffffffffu, gone != 0);
     if ((CONV || split) && !gave_up) {
       Tiles v(S, flags, digits, L::halves && split ? pass : -1);
@@ -1666,7 +1667,8 @@ int shift_mma_route(const GemmParams* ps, int n, bool conv, bool bound) {
   }
   if (terms < (conv ? 67108864.0 : 134217728.0)) return DS_ROUTE_CUDA_CORES;
   if (col_tiles > kMaxColTiles || tiles > INT32_MAX / kMaxCluster) return DS_ROUTE_CUDA_CORES;
-  if (conv && !bound && few_columns && terms >= (ps[0].R * ps[0].S <= 9 ? 134217728.0 : 189812531.0)) return DS_ROUTE_CUDA_CORES;
+  if (conv && !bound && few_columns && terms >= (ps[0].R * ps[0].S <= 9 ? 134217728.0 : 189812531.0))
+    return DS_ROUTE_CUDA_CORES;
   if (conv) return DS_ROUTE_TENSOR_CORES;
   const int64_t rows = ps[0].rows, cols = ps[0].cols;
   const int64_t pair_tiles = (rows + 2 * kRows - 1) / (2 * kRows) * ((cols + 127) / 128);
@@ -1685,7 +1687,8 @@ bool shift_mma_preferred(const GemmParams* ps, int n, bool conv) {
 
 cudaError_t launch_shift_mma(const GemmParams* ps, int n, bool conv, cudaStream_t st) {
   const bool bound = ps[0].amax_in != nullptr;
-  if (shift_mma_route(ps, n, conv, bound) == DS_ROUTE_TENSOR_CORES_SWAPPED) return launch_set<64, false>(ps, n, false, st);
+  if (shift_mma_route(ps, n, conv, bound) == DS_ROUTE_TENSOR_CORES_SWAPPED)
+    return launch_set<64, false>(ps, n, false, st);  // columns as lanes
   int64_t cols = 0;
   for (int i = 0; i < n; ++i) cols = std::max(cols, ps[i].cols);
   return cols <= 64 || (conv && !bound) ? launch_set<64, true>(ps, n, conv, st) : launch_set<128, true>(ps, n, conv, st);
